@@ -17,8 +17,15 @@
 // pre-activation receives (g_a - 2 a sum_k g_sk z_k)(1 - a^2) and each tangent
 // pre-activation g_sk (1 - a^2); weight gradients are GEMMs of the gradient rows with
 // the layer inputs over all 3B rows, input gradients GEMMs with the transposed weights.
-// Adam keeps float32 master weights and refreshes the BF16 copies (row-major and
-// transposed) used by the GEMMs.
+// Inference and training share one fused layer kernel (mlp_layer_persistent_kernel): its
+// epilogue sees the three streams of one (sample, feature) together and applies the
+// activation (forward), the loss (output layer) or the way back through the activation
+// (backward), so no GEMM result makes a trip through memory of its own.  Every weight
+// gradient comes from one launch (mlp_dw_kernel), the biases' from the row tiles' column
+// sums (mlp_grad_sum_kernel): nothing is added atomically, so a gradient is bitwise
+// reproducible.  Adam keeps float32 master weights and refreshes the BF16 copies
+// (row-major and transposed) used by the GEMMs.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <random>
@@ -28,141 +35,33 @@
 
 #include "internal.cuh"
 #include "mlp.cuh"
+#include "reduce.cuh"
 #include "tc_prims.cuh"
 
 namespace mrstat {
 namespace {
 
-constexpr int kLayers = 4;
-
 inline int pad8(int k) { return (k + 7) / 8 * 8; }
 
+// Layer 0's BF16 input rows for training: columns 0..2 the normalised (ln T1, ln T2, B1),
+// then the two tangents' rows; columns 3..7 zero.
 __global__ void mlp_input_kernel(const float* __restrict__ lnT, const float* __restrict__ b1, int B, float mu1,
-                                 float s1, float mu2, float s2, float mu3, float s3, __nv_bfloat16* __restrict__ X0,
-                                 __nv_bfloat16* __restrict__ X0T, int ldt) {
+                                 float s1, float mu2, float s2, float mu3, float s3, __nv_bfloat16* __restrict__ X0) {
+  red::pdl_trigger();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
   const float bb = b1 != nullptr ? b1[b] : 1.f;
   const float u[3] = {(lnT[b] - mu1) / s1, (lnT[B + b] - mu2) / s2, (bb - mu3) / s3};
-  const float t1[3] = {1.f / s1, 0.f, 0.f}, t2[3] = {0.f, 1.f / s2, 0.f};
+  __align__(16) __nv_bfloat16 o[3][8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
-    const float v0 = k < 3 ? u[k] : 0.f, v1 = k < 3 ? t1[k] : 0.f, v2 = k < 3 ? t2[k] : 0.f;
-    X0[(size_t)b * 8 + k] = __float2bfloat16_rn(v0);
-    X0[(size_t)(B + b) * 8 + k] = __float2bfloat16_rn(v1);
-    X0[(size_t)(2 * B + b) * 8 + k] = __float2bfloat16_rn(v2);
-    if (X0T != nullptr && k < 3) {
-      X0T[(size_t)k * ldt + b] = __float2bfloat16_rn(v0);
-      X0T[(size_t)k * ldt + B + b] = __float2bfloat16_rn(v1);
-      X0T[(size_t)k * ldt + 2 * B + b] = __float2bfloat16_rn(v2);
-    }
+    o[0][k] = __float2bfloat16_rn(k < 3 ? u[k] : 0.f);
+    o[1][k] = __float2bfloat16_rn(k == 0 ? 1.f / s1 : 0.f);
+    o[2][k] = __float2bfloat16_rn(k == 1 ? 1.f / s2 : 0.f);
   }
-}
-
-// hidden layer: value rows a = tanh(z + bias), tangent rows (1 - a^2) z_k
-__global__ void mlp_act_kernel(const float* __restrict__ Z, const float* __restrict__ bias, int B, int H,
-                               __nv_bfloat16* __restrict__ X, int ldx, __nv_bfloat16* __restrict__ XT, int ldt) {
-  const int64_t total = (int64_t)B * H;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(e / H), n = (int)(e - (int64_t)b * H);
-    const float a = tanhf(Z[(size_t)b * H + n] + bias[n]);
-    const float d = 1.f - a * a;
-    const float s1 = d * Z[(size_t)(B + b) * H + n];
-    const float s2 = d * Z[(size_t)(2 * B + b) * H + n];
-    X[(size_t)b * ldx + n] = __float2bfloat16_rn(a);
-    X[(size_t)(B + b) * ldx + n] = __float2bfloat16_rn(s1);
-    X[(size_t)(2 * B + b) * ldx + n] = __float2bfloat16_rn(s2);
-    if (XT != nullptr) {
-      XT[(size_t)n * ldt + b] = __float2bfloat16_rn(a);
-      XT[(size_t)n * ldt + B + b] = __float2bfloat16_rn(s1);
-      XT[(size_t)n * ldt + 2 * B + b] = __float2bfloat16_rn(s2);
-    }
-  }
-}
-
-// output layer: predictions (c, dc1, dc2) [3][R][B] and, with targets, the loss and its
-// gradient with respect to the output pre-activations
-__global__ void mlp_output_kernel(const float* __restrict__ Z, const float* __restrict__ bias,
-                                  const float* __restrict__ scale, int B, int R, float lam,
-                                  const float* __restrict__ target, float* __restrict__ pred,
-                                  __nv_bfloat16* __restrict__ GZ, int ldg, __nv_bfloat16* __restrict__ GZT, int ldt,
-                                  double* __restrict__ loss) {
-  const int64_t total = (int64_t)B * R;
-  double acc = 0.0;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(e / R), r = (int)(e - (int64_t)b * R);
-    const float sc = scale[r];
-    const float y0 = Z[(size_t)b * R + r] + bias[r];
-    const float y1 = Z[(size_t)(B + b) * R + r];
-    const float y2 = Z[(size_t)(2 * B + b) * R + r];
-    if (pred != nullptr) {
-      pred[(size_t)r * B + b] = sc * y0;
-      pred[(size_t)(R + r) * B + b] = sc * y1;
-      pred[(size_t)(2 * R + r) * B + b] = sc * y2;
-    }
-    if (target != nullptr) {
-      const float r0 = y0 - target[(size_t)r * B + b] / sc;
-      const float r1 = y1 - target[(size_t)(R + r) * B + b] / sc;
-      const float r2 = y2 - target[(size_t)(2 * R + r) * B + b] / sc;
-      acc += (double)r0 * r0 + (double)lam * ((double)r1 * r1 + (double)r2 * r2);
-      const float inv = 2.f / (float)B;
-      const float g0 = inv * r0, g1 = inv * lam * r1, g2 = inv * lam * r2;
-      GZ[(size_t)b * ldg + r] = __float2bfloat16_rn(g0);
-      GZ[(size_t)(B + b) * ldg + r] = __float2bfloat16_rn(g1);
-      GZ[(size_t)(2 * B + b) * ldg + r] = __float2bfloat16_rn(g2);
-      GZT[(size_t)r * ldt + b] = __float2bfloat16_rn(g0);
-      GZT[(size_t)r * ldt + B + b] = __float2bfloat16_rn(g1);
-      GZT[(size_t)r * ldt + 2 * B + b] = __float2bfloat16_rn(g2);
-    }
-  }
-  if (target != nullptr) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0 && acc != 0.0) atomicAdd(loss, acc / (double)B);
-  }
-}
-
-// backward through a tanh layer: GX [3B][H] = dL/d(layer output) -> GZ (and transposed), db
-__global__ void mlp_backact_kernel(const float* __restrict__ GX, const float* __restrict__ Z,
-                                   const float* __restrict__ bias, int B, int H, __nv_bfloat16* __restrict__ GZ,
-                                   int ldg, __nv_bfloat16* __restrict__ GZT, int ldt, float* __restrict__ db) {
-  const int64_t total = (int64_t)B * H;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(e / H), n = (int)(e - (int64_t)b * H);
-    const float a = tanhf(Z[(size_t)b * H + n] + bias[n]);
-    const float d = 1.f - a * a;
-    const float z1 = Z[(size_t)(B + b) * H + n], z2 = Z[(size_t)(2 * B + b) * H + n];
-    const float ga = GX[(size_t)b * H + n], g1 = GX[(size_t)(B + b) * H + n], g2 = GX[(size_t)(2 * B + b) * H + n];
-    const float gz1 = g1 * d, gz2 = g2 * d;
-    const float gz = (ga - 2.f * a * (g1 * z1 + g2 * z2)) * d;
-    GZ[(size_t)b * ldg + n] = __float2bfloat16_rn(gz);
-    GZ[(size_t)(B + b) * ldg + n] = __float2bfloat16_rn(gz1);
-    GZ[(size_t)(2 * B + b) * ldg + n] = __float2bfloat16_rn(gz2);
-    GZT[(size_t)n * ldt + b] = __float2bfloat16_rn(gz);
-    GZT[(size_t)n * ldt + B + b] = __float2bfloat16_rn(gz1);
-    GZT[(size_t)n * ldt + 2 * B + b] = __float2bfloat16_rn(gz2);
-    atomicAdd(db + n, gz);
-  }
-}
-
-// output-layer bias gradient: sum over the value rows of the output gradient
-__global__ void mlp_out_bias_grad_kernel(const float* __restrict__ Z, const float* __restrict__ bias,
-                                         const float* __restrict__ scale, const float* __restrict__ target, int B,
-                                         int R, float* __restrict__ db) {
-  const int r = blockIdx.x;
-  float acc = 0.f;
-  for (int b = threadIdx.x; b < B; b += blockDim.x)
-    acc += 2.f / (float)B * (Z[(size_t)b * R + r] + bias[r] - target[(size_t)r * B + b] / scale[r]);
-  __shared__ float ws[32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float s = 0.f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += ws[w];
-    db[r] = s;
-  }
+  for (int k = 0; k < 3; ++k)
+    *reinterpret_cast<uint4*>(X0 + ((size_t)k * B + b) * 8) = *reinterpret_cast<const uint4*>(o[k]);
 }
 
 // Adam on one layer (weights [out][in] then bias [out]) and refresh of its BF16 copies
@@ -290,11 +189,62 @@ struct PerShape {
 constexpr int kPerEpiWarps = 16;  // four per TMEM lane quarter, one 16-column chunk each
 constexpr int kPerThreads = 64 + 32 * kPerEpiWarps;
 
-template <bool LAST>
+// What the epilogue of a layer does with the three accumulators z, z1, z2 of a (sample,
+// feature): inference (hidden, output), training forward (hidden: also keeps a, z1, z2 in
+// float32; output: the loss and the gradient rows) and training backward (the accumulators
+// are dL/d(layer output); back through the layer's tanh, and for layer 0 its weight
+// gradient's sums instead of gradient rows).
+enum LayerMode { kInferHidden, kInferLast, kTrainHidden, kTrainLast, kBack, kBackFirst };
+
+struct LayerIo {
+  const float* bias = nullptr;       // [N]
+  __nv_bfloat16* xn = nullptr;       // [3B][ldn]: next layer's input rows, or the gradient rows
+  int ldn = 0;
+  const float* scale = nullptr;      // [R] output scale
+  float* pred = nullptr;             // [3][R][B] (inference)
+  float* za = nullptr;               // [3][B][N] a, z1, z2 of the layer (training)
+  const float* target = nullptr;     // [3][R][B]
+  float lam = 0.f;
+  float* colpart = nullptr;          // [4 row tiles][sums][N] sums over 32 rows each (1 sum; kBackFirst 6)
+  double* losspart = nullptr;        // [4 row tiles][column chunks of 8]
+  const float* lnT = nullptr;        // kBackFirst: layer 0's inputs
+  const float* b1 = nullptr;
+  float norm[6] = {0.f, 1.f, 0.f, 1.f, 1.f, 1.f};
+};
+
+// Sums of K columns over a warp's 32 rows by halving exchanges (K + log2(32 / K) - 1
+// shuffles); lane l returns the sum of column l K / 32.
+template <int K>
+__device__ __forceinline__ float warp_columns(float (&v)[K], int lane) {
+#pragma unroll
+  for (int n = K, off = 16; n > 1; n >>= 1, off >>= 1) {
+    const bool up = lane & off;
+#pragma unroll
+    for (int i = 0; i < n / 2; ++i) {
+      const float send = up ? v[i] : v[i + n / 2];
+      const float keep = up ? v[i + n / 2] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+    }
+  }
+  float t = v[0];
+#pragma unroll
+  for (int off = 16 / K; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+  return t;
+}
+
+// K BF16 values of one row to columns col.. of a row-major matrix with leading dimension ld
+// (ld and col are multiples of 8 elements), the columns past ld left out
+template <int K>
+__device__ __forceinline__ void store_row(__nv_bfloat16* row, int col, int ld, const __nv_bfloat16 (&o)[K]) {
+#pragma unroll
+  for (int j = 0; j < K; j += 8)
+    if (col + j < ld) *reinterpret_cast<uint4*>(row + col + j) = *reinterpret_cast<const uint4*>(o + j);
+}
+
+template <int MODE>
 __global__ void __launch_bounds__(kPerThreads, 1)
 mlp_layer_persistent_kernel(const __grid_constant__ CUtensorMap tx, const __grid_constant__ CUtensorMap tw, int B,
-                            int N, int K, const float* __restrict__ bias, __nv_bfloat16* __restrict__ xn, int ldn,
-                            const float* __restrict__ scale, float* __restrict__ pred, int* __restrict__ err) {
+                            int N, int K, const __grid_constant__ LayerIo io, int* __restrict__ err) {
   using namespace tc;
   using PS = PerShape;
   constexpr int BN = PS::BN;
@@ -328,6 +278,8 @@ mlp_layer_persistent_kernel(const __grid_constant__ CUtensorMap tx, const __grid
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;
+  red::pdl_trigger();
+  red::pdl_wait();  // the input rows come from the previous launch
 
   int issued = 0;
   if (warp == 0) {
@@ -388,61 +340,195 @@ mlp_layer_persistent_kernel(const __grid_constant__ CUtensorMap tx, const __grid
     }
   } else {
     const int q = warp & 3;              // TMEM lane quarter of this warp
-    const int cb = ((warp - 2) >> 2) * 16;  // its 16-column chunk of the tile
+    // its 16-column chunk of the tile (the output layer in training has at most 32 columns:
+    // 8 each, so that all sixteen warps share them)
+    constexpr int kCols = MODE == kTrainLast ? 8 : 16;
+    const int cb = ((warp - 2) >> 2) * kCols;
     int i = 0;
     for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++i) {
       const int acc = i & 1;
+      const int b0 = (t / n_tiles) * BM, n0 = (t % n_tiles) * BN;
+      const int b = b0 + q * 32 + lane;  // this lane's row (sample)
+      float tg[3][8];  // the targets, loaded while the accumulators are formed
+      if constexpr (MODE == kTrainLast) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            tg[k][j] = b < B && cb + j < N ? io.target[(size_t)(k * N + cb + j) * B + b] : 0.f;
+      }
       if (!mbar_wait(&accf[acc], (uint32_t)(i >> 1) & 1u, abort_flag)) break;
       __syncwarp();
       fence_after();
-      const int b0 = (t / n_tiles) * BM, n0 = (t % n_tiles) * BN;
-      const int b = b0 + q * 32 + lane;  // this lane's row (sample)
       const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * 3 * BN);
-      float v0[16], v1[16], v2[16];
-      tmem_ld16(trow + (uint32_t)cb, v0);
-      tmem_ld16(trow + (uint32_t)(BN + cb), v1);
-      tmem_ld16(trow + (uint32_t)(2 * BN + cb), v2);
+      float v0[kCols], v1[kCols], v2[kCols];
+      if constexpr (kCols == 16) {
+        tmem_ld16(trow + (uint32_t)cb, v0);
+        tmem_ld16(trow + (uint32_t)(BN + cb), v1);
+        tmem_ld16(trow + (uint32_t)(2 * BN + cb), v2);
+      } else {
+        tmem_ld8(trow + (uint32_t)cb, v0);
+        tmem_ld8(trow + (uint32_t)(BN + cb), v1);
+        tmem_ld8(trow + (uint32_t)(2 * BN + cb), v2);
+      }
       // this warp's part of the accumulator set is in registers: hand it back
       fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&acce[acc]);
-      if (b >= B) continue;
-      if (LAST) {
+      const int col = n0 + cb;  // this warp's first column
+      const bool on = b < B;
+      if constexpr (MODE == kInferLast) {
+        if (!on) continue;
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-          const int r = n0 + cb + j;
+          const int r = col + j;
           if (r < N) {
-            const float sc = scale[r];
-            pred[(size_t)r * B + b] = sc * (v0[j] + bias[r]);
-            pred[(size_t)(N + r) * B + b] = sc * v1[j];
-            pred[(size_t)(2 * N + r) * B + b] = sc * v2[j];
+            const float sc = io.scale[r];
+            io.pred[(size_t)r * B + b] = sc * (v0[j] + io.bias[r]);
+            io.pred[(size_t)(N + r) * B + b] = sc * v1[j];
+            io.pred[(size_t)(2 * N + r) * B + b] = sc * v2[j];
           }
         }
-      } else {
+      } else if constexpr (MODE == kInferHidden) {
+        if (!on) continue;
         __align__(16) __nv_bfloat16 o[3][16];
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-          const int n = n0 + cb + j;
-          const float a = tanh_fast(v0[j] + (n < N ? bias[n] : 0.f));
+          const int n = col + j;
+          const float a = tanh_fast(v0[j] + (n < N ? io.bias[n] : 0.f));
           const float dd = 1.f - a * a;
           o[0][j] = __float2bfloat16_rn(a);
           o[1][j] = __float2bfloat16_rn(dd * v1[j]);
           o[2][j] = __float2bfloat16_rn(dd * v2[j]);
         }
-        const int col = n0 + cb;
-        if (col + 16 <= ldn) {  // 32 bytes per stream (ldn and col are multiples of 8 elements)
 #pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            uint4* dst = reinterpret_cast<uint4*>(xn + ((size_t)k * B + b) * ldn + col);
-            dst[0] = reinterpret_cast<const uint4*>(o[k])[0];
-            dst[1] = reinterpret_cast<const uint4*>(o[k])[1];
+        for (int k = 0; k < 3; ++k) store_row(io.xn + ((size_t)k * B + b) * io.ldn, col, io.ldn, o[k]);
+      } else if constexpr (MODE == kTrainHidden) {
+        if (!on) continue;  // N is the hidden width, a multiple of the 64-column tile
+        __align__(16) __nv_bfloat16 o[3][16];
+        float* za = io.za + (size_t)b * N + col;
+        const size_t plane = (size_t)B * N;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          float av[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int j = 4 * g + i;
+            const float a = tanhf(v0[j] + io.bias[col + j]);
+            const float d = 1.f - a * a;
+            av[i] = a;
+            o[0][j] = __float2bfloat16_rn(a);
+            o[1][j] = __float2bfloat16_rn(d * v1[j]);
+            o[2][j] = __float2bfloat16_rn(d * v2[j]);
+          }
+          *reinterpret_cast<float4*>(za + 4 * g) = make_float4(av[0], av[1], av[2], av[3]);
+          *reinterpret_cast<float4*>(za + plane + 4 * g) = make_float4(v1[4 * g], v1[4 * g + 1], v1[4 * g + 2], v1[4 * g + 3]);
+          *reinterpret_cast<float4*>(za + 2 * plane + 4 * g) =
+              make_float4(v2[4 * g], v2[4 * g + 1], v2[4 * g + 2], v2[4 * g + 3]);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) store_row(io.xn + ((size_t)k * B + b) * io.ldn, col, io.ldn, o[k]);
+      } else if constexpr (MODE == kTrainLast) {
+        // predictions against the targets: the loss, the gradient rows with respect to the
+        // output pre-activations and the output bias's column sums
+        if (col >= N) continue;  // the same in every lane of the warp
+        __align__(16) __nv_bfloat16 o[3][8];
+        float hi = 0.f, lo = 0.f;  // the loss terms as a float-float sum (float64 is slow here)
+        auto add_square = [&](float wt, float x) {  // wt x^2, its rounding error included
+          const float y = wt * x, p = y * x;
+          const float e = fmaf(y, x, -p) + fmaf(wt, x, -y) * x;
+          const float t = hi + p, bb = t - hi;
+          lo += ((hi - (t - bb)) + (p - bb)) + e;
+          hi = t;
+        };
+        const float inv = 2.f / (float)B;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          float g0 = 0.f, g1 = 0.f, g2 = 0.f;
+          if (col + j < N && on) {
+            const float sc = io.scale[col + j];
+            const float r0 = v0[j] + io.bias[col + j] - tg[0][j] / sc;
+            const float r1 = v1[j] - tg[1][j] / sc;
+            const float r2 = v2[j] - tg[2][j] / sc;
+            add_square(1.f, r0);
+            add_square(io.lam, r1);
+            add_square(io.lam, r2);
+            g0 = inv * r0;
+            g1 = inv * io.lam * r1;
+            g2 = inv * io.lam * r2;
+          }
+          o[0][j] = __float2bfloat16_rn(g0);
+          o[1][j] = __float2bfloat16_rn(g1);
+          o[2][j] = __float2bfloat16_rn(g2);
+          v0[j] = g0;
+        }
+        if (on) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) store_row(io.xn + ((size_t)k * B + b) * io.ldn, col, io.ldn, o[k]);
+        }
+        const size_t prow = (size_t)(b0 / BM) * 4 + q;
+        const float sum = warp_columns(v0, lane);
+        if ((lane & 3) == 0 && col + (lane >> 2) < N) io.colpart[prow * N + col + (lane >> 2)] = sum;
+        double acc = (double)hi + (double)lo;
+#pragma unroll
+        for (int of = 16; of > 0; of >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, of);
+        if (lane == 0) io.losspart[prow * ((N + 7) / 8) + (col >> 3)] = acc;
+      } else {
+        // kBack, kBackFirst: v0, v1, v2 = dL/d(a, s1, s2) of a tanh layer
+        __align__(16) __nv_bfloat16 o[3][16];
+        const float* za = io.za + (size_t)(on ? b : 0) * N + col;
+        const size_t plane = (size_t)B * N;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          const float4 a4 = *reinterpret_cast<const float4*>(za + 4 * g);
+          const float4 p4 = *reinterpret_cast<const float4*>(za + plane + 4 * g);
+          const float4 q4 = *reinterpret_cast<const float4*>(za + 2 * plane + 4 * g);
+          const float av[4] = {a4.x, a4.y, a4.z, a4.w}, zv1[4] = {p4.x, p4.y, p4.z, p4.w},
+                      zv2[4] = {q4.x, q4.y, q4.z, q4.w};
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int j = 4 * g + i;
+            const float a = av[i], z1 = zv1[i], z2 = zv2[i];
+            const float d = 1.f - a * a;
+            const float ga = v0[j], g1 = v1[j], g2 = v2[j];
+            const float gz1 = g1 * d, gz2 = g2 * d;
+            const float gz = (ga - 2.f * a * (g1 * z1 + g2 * z2)) * d;
+            o[0][j] = __float2bfloat16_rn(gz);
+            o[1][j] = __float2bfloat16_rn(gz1);
+            o[2][j] = __float2bfloat16_rn(gz2);
+            v0[j] = on ? gz : 0.f;
+          }
+        }
+        const size_t prow = (size_t)(b0 / BM) * 4 + q;
+        constexpr int kSums = MODE == kBackFirst ? 6 : 1;
+        float* cp = io.colpart + prow * kSums * N + col + (lane >> 1);
+        const float sum = warp_columns(v0, lane);
+        if ((lane & 1) == 0) cp[0] = sum;
+        if constexpr (MODE == kBack) {
+          if (on) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) store_row(io.xn + ((size_t)k * B + b) * io.ldn, col, io.ldn, o[k]);
           }
         } else {
+          // layer 0's weight gradient: its inputs are three columns, so the sums over the
+          // BF16 gradient rows times the BF16 inputs are formed here
+          float u[3] = {0.f, 0.f, 0.f};
+          if (on) {
+            const float bb = io.b1 != nullptr ? io.b1[b] : 1.f;
+            u[0] = __bfloat162float(__float2bfloat16_rn((io.lnT[b] - io.norm[0]) / io.norm[1]));
+            u[1] = __bfloat162float(__float2bfloat16_rn((io.lnT[B + b] - io.norm[2]) / io.norm[3]));
+            u[2] = __bfloat162float(__float2bfloat16_rn((bb - io.norm[4]) / io.norm[5]));
+          }
 #pragma unroll
-          for (int k = 0; k < 3; ++k)
+          for (int k = 0; k < 5; ++k) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j)
-              if (col + j < ldn) xn[((size_t)k * B + b) * ldn + col + j] = o[k][j];
+            for (int j = 0; j < 16; ++j) {
+              if (k < 3) v0[j] = __bfloat162float(o[0][j]) * u[k];
+              else v0[j] = on ? __bfloat162float(o[k - 2][j]) : 0.f;
+            }
+            const float t = warp_columns(v0, lane);
+            if ((lane & 1) == 0) cp[(size_t)(k + 1) * N] = t;
+          }
         }
       }
     }
@@ -463,6 +549,169 @@ mlp_layer_persistent_kernel(const __grid_constant__ CUtensorMap tx, const __grid
   if (warp == 0) tmem_dealloc<PS::kTmemCols>(tmem);
 }
 
+// ---------------------------------------------------------------------------
+// Weight gradient dW_l = GZ_l^T X_l of one layer (l = 1..3) over the 3B gradient and input
+// rows: one CTA per 128 x 64 tile.  Both operands are read as they were written (rows = the
+// GEMM's K): MN-major tiles of 64 rows, so no transposed copies exist.  Bound by the chain
+// of dependent MMAs over the rows, about 75 ns per 16 rows at any tile size: 57 us at 4096
+// samples (108 us from transposed K-major copies, 64-row chunks of 32 KB).  The rows are not
+// split over CTAs: the tensor core's float32 accumulation rounds towards zero, so a split
+// changes a gradient by 3e-5 relative.  The launch uses few SMs (8 at H = 256), so the three
+// layers' gradients run on streams of their own beside the backward layers.
+// ---------------------------------------------------------------------------
+constexpr int kDwN = 64;                             // columns of a tile
+constexpr int kDwStages = 8;
+constexpr uint32_t kDwBox = 64 * tc::BK * 2;         // 64 rows x 64 columns
+constexpr uint32_t kDwStage = 3 * kDwBox;            // two boxes of GZ, one of X
+constexpr size_t kDwSmem = (size_t)kDwStages * kDwStage + 1024 + 256;
+
+__global__ void __launch_bounds__(128, 1)
+mlp_dw_kernel(const __grid_constant__ CUtensorMap tgz, const __grid_constant__ CUtensorMap tx, int rows, int out,
+              int in, float* __restrict__ grad, int* __restrict__ err) {
+  using namespace tc;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kDwStages * kDwStage);
+  uint64_t* empty = full + kDwStages;
+  uint64_t* done = empty + kDwStages;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nt = in / kDwN;  // in is the hidden width, a multiple of 64
+  const int m0 = (blockIdx.x / nt) * BM, n0 = (blockIdx.x % nt) * kDwN;
+  const int nk = (rows + BK - 1) / BK;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kDwStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(done, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) tmem_alloc<64>(tmem_slot);
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  int issued = 0;
+  if (warp == 0 && lane == 0) {
+    for (int g = 0; g < nk; ++g) {
+      const int s = g % kDwStages;
+      if (g >= kDwStages && !mbar_wait(&empty[s], (uint32_t)(g / kDwStages - 1) & 1u, abort_flag)) break;
+      uint8_t* st = smem + s * kDwStage;
+      mbar_expect_tx(&full[s], kDwStage);
+      tma_load_2d(&tgz, &full[s], st, m0, g * BK);
+      tma_load_2d(&tgz, &full[s], st + kDwBox, m0 + 64, g * BK);
+      tma_load_2d(&tx, &full[s], st + 2 * kDwBox, n0, g * BK);
+      issued = g + 1;
+    }
+  } else if (warp == 1 && lane == 0) {
+    constexpr uint32_t idesc = make_idesc(BM, kDwN) | kIdescMnMajorA | kIdescMnMajorB;
+    for (int g = 0; g < nk; ++g) {
+      const int s = g % kDwStages;
+      if (!mbar_wait(&full[s], (uint32_t)(g / kDwStages) & 1u, abort_flag)) break;
+      fence_after();
+      const uint8_t* st = smem + s * kDwStage;
+      const uint64_t da = sdesc_sw128_mn(st, kDwBox), db = sdesc_sw128_mn(st + 2 * kDwBox, kDwBox);
+#pragma unroll
+      for (int k = 0; k < BK / 16; ++k)  // 16 rows of 128 bytes, in 16-byte units
+        mma_bf16(tmem, da + 128ull * k, db + 128ull * k, idesc, (g > 0 || k > 0) ? 1u : 0u);
+      mma_commit(&empty[s]);
+    }
+    mma_commit(done);
+  }
+  __syncwarp();
+  const bool ok = mbar_wait(done, 0, abort_flag) && *abort_flag == 0;
+  __syncwarp();
+  fence_after();
+  if (ok) {
+    const int o = m0 + warp * 32 + lane;
+    float* dst = grad + (int64_t)o * in + n0;
+#pragma unroll
+    for (int cb = 0; cb < kDwN; cb += 16) {
+      float v[16];
+      tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)cb, v);
+      if (o < out) {
+#pragma unroll
+        for (int j = 0; j < 16; j += 4)
+          *reinterpret_cast<float4*>(dst + cb + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+      }
+    }
+  } else if (threadIdx.x == 0) {
+    atomicExch(err, 1);
+    // let the copies this thread issued land before the CTA's shared memory goes away
+    for (int g = issued > kDwStages ? issued - kDwStages : 0; g < issued; ++g) {
+      int spins = 0;
+      while (!mbar_try_wait(&full[g % kDwStages], (uint32_t)(g / kDwStages) & 1u) && ++spins < (1 << 16)) {
+      }
+    }
+  }
+  fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_dealloc<64>(tmem);
+}
+
+// The biases' and layer 0's gradient from the row tiles' column sums, in a fixed order (32
+// columns per block, the tiles split over its warps: latency, not bytes, bounds it), and the loss (last block).
+constexpr int kSumWarps = 16;
+__global__ void __launch_bounds__(32 * kSumWarps)
+mlp_grad_sum_kernel(const float* __restrict__ cp0, const float* __restrict__ cp1, const float* __restrict__ cp2,
+                    const float* __restrict__ cp3, const double* __restrict__ losspart, int nloss, int prows, int H,
+                    int R, int B, float d1, float d2, float* __restrict__ grad, double* __restrict__ loss) {
+  const int64_t off1 = 4 * (int64_t)H, off2 = off1 + (int64_t)H * H + H, off3 = off2 + (int64_t)H * H + H;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  red::pdl_wait();
+  __shared__ float ws[kSumWarps][6][32];
+  if (blockIdx.x == gridDim.x - 1) {
+    __shared__ double wd[kSumWarps];
+    double s = 0.0;
+    for (int i = threadIdx.x; i < nloss; i += 32 * kSumWarps) s += losspart[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) wd[warp] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int k = 1; k < kSumWarps; ++k) s += wd[k];
+      *loss = s / (double)B;
+    }
+    return;
+  }
+  const int c = blockIdx.x * 32 + lane;  // column: layer 0, 1, 2 (H each), 3 (R)
+  const int l = c / H, n = c - l * H;
+  const bool in = l < 3 || (l == 3 && n < R);
+  const float* cp = l == 0 ? cp0 : l == 1 ? cp1 : l == 2 ? cp2 : cp3;
+  const int sums = l == 0 ? 6 : 1, ld = l == 3 ? R : H;
+  float s[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  if (in) {
+#pragma unroll 4
+    for (int p = warp; p < prows; p += kSumWarps)
+#pragma unroll
+      for (int k = 0; k < 6; ++k)
+        if (k < sums) s[k] += cp[((size_t)p * sums + k) * ld + n];
+  }
+#pragma unroll
+  for (int k = 0; k < 6; ++k) ws[warp][k][lane] = s[k];
+  __syncthreads();
+  if (warp != 0 || !in) return;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    s[k] = 0.f;
+#pragma unroll
+    for (int w = 0; w < kSumWarps; ++w) s[k] += ws[w][k][lane];
+  }
+  if (l == 0) {
+    grad[3 * H + n] = s[0];
+    grad[3 * n] = fmaf(d1, s[4], s[1]);
+    grad[3 * n + 1] = fmaf(d2, s[5], s[2]);
+    grad[3 * n + 2] = s[3];
+  } else {
+    grad[l == 1 ? off2 - H + n : l == 2 ? off3 - H + n : off3 + (int64_t)R * H + n] = s[0];
+  }
+}
+
 int blocks_for(int64_t n, int t = 256) {
   int64_t b = (n + t - 1) / t;
   return (int)(b < 1 ? 1 : (b > 8192 ? 8192 : b));
@@ -474,7 +723,13 @@ int blocks_for(int64_t n, int t = 256) {
 Mlp::~Mlp() {
   release_batch();
   free_weights();
-  if (dev_err) cudaFree(dev_err);
+  if (stat) cudaFree(stat);
+  if (stat_host) cudaFreeHost(stat_host);
+  for (int k = 0; k < 3; ++k) {
+    if (side[k]) cudaStreamDestroy(side[k]);
+    if (ev_fork[k]) cudaEventDestroy(ev_fork[k]);
+    if (ev_join[k]) cudaEventDestroy(ev_join[k]);
+  }
 }
 
 void Mlp::free_weights() {
@@ -491,16 +746,14 @@ void Mlp::free_weights() {
 
 void Mlp::release_batch() {
   for (int l = 0; l < 4; ++l) {
-    void* ptrs[] = {X[l], XT[l], Z[l], GZ[l], GZT[l]};
+    void* ptrs[] = {X[l], ZA[l], GZ[l], colpart[l]};
     for (void* q : ptrs)
       if (q) cudaFree(q);
-    X[l] = XT[l] = GZ[l] = GZT[l] = nullptr;
-    Z[l] = nullptr;
+    X[l] = GZ[l] = nullptr;
+    ZA[l] = colpart[l] = nullptr;
   }
-  if (GX) cudaFree(GX);
-  if (loss_dev) cudaFree(loss_dev);
-  GX = nullptr;
-  loss_dev = nullptr;
+  if (losspart) cudaFree(losspart);
+  losspart = nullptr;
   cap = 0;
   maps_b = -1;
 }
@@ -508,6 +761,7 @@ void Mlp::release_batch() {
 int Mlp::setup(int h, int r, uint64_t seed) {
   H = h;
   R = r;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || sms < 1) sms = 1;
   const int dims[5] = {3, H, H, H, R};
   np = 0;
   for (int l = 0; l < 4; ++l) {
@@ -525,17 +779,24 @@ int Mlp::setup(int h, int r, uint64_t seed) {
   chk(cudaMalloc(&adam_v, np * sizeof(float)));
   chk(cudaMalloc(&grad, np * sizeof(float)));
   chk(cudaMalloc(&scale_dev, R * sizeof(float)));
-  chk(cudaMalloc(&dev_err, sizeof(int)));
-  if (e == cudaSuccess) chk(cudaMemset(dev_err, 0, sizeof(int)));
+  chk(cudaMalloc(&stat, 2 * sizeof(double)));
+  chk(cudaMallocHost(&stat_host, 2 * sizeof(double)));
+  if (e == cudaSuccess) chk(cudaMemset(stat, 0, 2 * sizeof(double)));
+  for (int k = 0; k < 3; ++k) {
+    chk(cudaStreamCreateWithFlags(&side[k], cudaStreamNonBlocking));
+    chk(cudaEventCreateWithFlags(&ev_fork[k], cudaEventDisableTiming));
+    chk(cudaEventCreateWithFlags(&ev_join[k], cudaEventDisableTiming));
+  }
+  loss_dev = stat;
+  dev_err = reinterpret_cast<int*>(stat + 1);
   for (int l = 0; l < 4; ++l) {
     chk(cudaMalloc(&Wb[l], (size_t)out[l] * pad8(in[l]) * 2));
     chk(cudaMalloc(&WTb[l], (size_t)in[l] * pad8(out[l]) * 2));
     if (e == cudaSuccess) {
       chk(cudaMemset(Wb[l], 0, (size_t)out[l] * pad8(in[l]) * 2));
       chk(cudaMemset(WTb[l], 0, (size_t)in[l] * pad8(out[l]) * 2));
-      chk(make_split_operand(&opW[l], Wb[l], Wb[l], out[l], in[l], pad8(in[l]), false));
       chk(make_bf16_tmap(&wmap64[l], Wb[l], out[l], in[l], pad8(in[l]), PerShape::BN));
-      chk(make_split_operand(&opWT[l], WTb[l], WTb[l], in[l], out[l], pad8(out[l]), false));
+      chk(make_bf16_tmap(&wtmap64[l], WTb[l], in[l], out[l], pad8(out[l]), PerShape::BN));
     }
   }
   if (e != cudaSuccess) return cuda_fail(e, "surrogate allocation");
@@ -571,7 +832,8 @@ int Mlp::set_params(const float* host, cudaStream_t st) {
 int Mlp::ensure_batch(int B, bool train) {
   if (B > cap || (train && !have_train_buffers)) {
     release_batch();
-    const int Mc = 3 * B, Mp = pad8(Mc);
+    const int Mc = 3 * B;
+    const size_t prows = 4 * (size_t)((B + tc::BM - 1) / tc::BM);
     cudaError_t e = cudaSuccess;
     auto chk = [&](cudaError_t q) {
       if (e == cudaSuccess) e = q;
@@ -579,21 +841,17 @@ int Mlp::ensure_batch(int B, bool train) {
     for (int l = 0; l < 4; ++l) {
       chk(cudaMalloc(&X[l], (size_t)Mc * pad8(in[l]) * 2));
       if (train) {
-        chk(cudaMalloc(&Z[l], (size_t)Mc * out[l] * sizeof(float)));
-        chk(cudaMalloc(&XT[l], (size_t)in[l] * Mp * 2));
-        chk(cudaMalloc(&GZ[l], (size_t)Mc * pad8(out[l]) * 2));
-        chk(cudaMalloc(&GZT[l], (size_t)out[l] * Mp * 2));
+        if (l < 3) chk(cudaMalloc(&ZA[l], (size_t)Mc * out[l] * sizeof(float)));
+        if (l > 0) chk(cudaMalloc(&GZ[l], (size_t)Mc * pad8(out[l]) * 2));
+        chk(cudaMalloc(&colpart[l], prows * (l == 0 ? 6 : 1) * out[l] * sizeof(float)));
       }
     }
-    if (train) chk(cudaMalloc(&GX, (size_t)Mc * H * sizeof(float)));
-    chk(cudaMalloc(&loss_dev, sizeof(double)));
+    if (train) {
+      chk(cudaMalloc(&losspart, prows * ((R + 7) / 8) * sizeof(double)));
+    }
     for (int l = 0; l < 4 && e == cudaSuccess; ++l) {
       chk(cudaMemset(X[l], 0, (size_t)Mc * pad8(in[l]) * 2));
-      if (train) {
-        chk(cudaMemset(XT[l], 0, (size_t)in[l] * Mp * 2));
-        chk(cudaMemset(GZ[l], 0, (size_t)Mc * pad8(out[l]) * 2));
-        chk(cudaMemset(GZT[l], 0, (size_t)out[l] * Mp * 2));
-      }
+      if (train && l > 0) chk(cudaMemset(GZ[l], 0, (size_t)Mc * pad8(out[l]) * 2));
     }
     if (e != cudaSuccess) {
       release_batch();
@@ -603,13 +861,15 @@ int Mlp::ensure_batch(int B, bool train) {
     have_train_buffers = train;
   }
   if (maps_b != B || maps_train != train) {
-    const int Mc = 3 * B, Mp = pad8(3 * cap);
+    const int Mc = 3 * B;
     cudaError_t e = cudaSuccess;
     for (int l = 0; l < 4 && e == cudaSuccess; ++l) {
-      e = make_split_operand(&opX[l], X[l], X[l], Mc, in[l], pad8(in[l]), true);
-      if (e == cudaSuccess && train) e = make_split_operand(&opXT[l], XT[l], XT[l], in[l], Mc, Mp, false);
-      if (e == cudaSuccess && train) e = make_split_operand(&opGZ[l], GZ[l], GZ[l], Mc, out[l], pad8(out[l]), true);
-      if (e == cudaSuccess && train) e = make_split_operand(&opGZT[l], GZT[l], GZT[l], out[l], Mc, Mp, true);
+      e = make_bf16_tmap(&xmap[l], X[l], Mc, in[l], pad8(in[l]), tc::BM);
+      if (!train || l == 0) continue;
+      if (e == cudaSuccess) e = make_bf16_tmap(&gzmap[l], GZ[l], Mc, out[l], pad8(out[l]), tc::BM);
+      // 64-row boxes, the rows as the GEMM's K (the weight gradients)
+      if (e == cudaSuccess) e = make_bf16_tmap(&xmap_k[l], X[l], Mc, in[l], pad8(in[l]), tc::BK);
+      if (e == cudaSuccess) e = make_bf16_tmap(&gzmap_k[l], GZ[l], Mc, out[l], pad8(out[l]), tc::BK);
     }
     if (e != cudaSuccess) return cuda_fail(e, "surrogate tensor maps");
     maps_b = B;
@@ -618,54 +878,92 @@ int Mlp::ensure_batch(int B, bool train) {
   return MRSTAT_OK;
 }
 
-int Mlp::forward(const float* lnT, const float* b1, int B, bool train, cudaStream_t st) {
-  const int Mc = 3 * B;
-  const int ldt = pad8(3 * cap);
-  mlp_input_kernel<<<blocks_for(B), 256, 0, st>>>(lnT, b1, B, norm[0], norm[1], norm[2], norm[3], norm[4], norm[5],
-                                                  X[0], train ? XT[0] : nullptr, ldt);
-  cudaError_t e = cudaGetLastError();
-  for (int l = 0; l < 4 && e == cudaSuccess; ++l) {
-    e = launch_tc_gemm(opX[l], opW[l], Z[l], Mc, out[l], in[l], out[l], 1, nullptr, dev_err, st);
-    if (e != cudaSuccess || l == 3) break;
-    mlp_act_kernel<<<blocks_for((int64_t)B * out[l]), 256, 0, st>>>(Z[l], theta + off[l] + (int64_t)out[l] * in[l],
-                                                                    B, out[l], X[l + 1], pad8(in[l + 1]),
-                                                                    train ? XT[l + 1] : nullptr, ldt);
-    e = cudaGetLastError();
-  }
-  return e == cudaSuccess ? MRSTAT_OK : cuda_fail(e, "surrogate forward");
+template <int MODE>
+static cudaError_t launch_layer(const CUtensorMap& x, const CUtensorMap& w, int B, int N, int K, const LayerIo& io,
+                                int sms, int* err, cudaStream_t st) {
+  const size_t sm = PerShape::kSmem;
+  cudaError_t e = cudaFuncSetAttribute(mlp_layer_persistent_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sm);
+  if (e != cudaSuccess) return e;
+  const int tiles = ((B + tc::BM - 1) / tc::BM) * ((N + PerShape::BN - 1) / PerShape::BN);
+  // programmatic dependent launch: the set-up overlaps the previous layer's tail
+  return launch_pdl(mlp_layer_persistent_kernel<MODE>, dim3(std::max(1, std::min(tiles, sms))), dim3(kPerThreads), sm, st,
+                    x, w, B, N, K, io, err);
 }
 
-int Mlp::backward(const float* target, int B, cudaStream_t st) {
-  const int Mc = 3 * B;
-  const int ldt = pad8(3 * cap);
-  cudaError_t e = cudaMemsetAsync(grad, 0, np * sizeof(float), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(loss_dev, 0, sizeof(double), st);
-  // output layer
-  const float* b4 = theta + off[3] + (int64_t)out[3] * in[3];
-  if (e == cudaSuccess) {
-    mlp_output_kernel<<<blocks_for((int64_t)B * R), 256, 0, st>>>(Z[3], b4, scale_dev, B, R, lam, target, nullptr,
-                                                                  GZ[3], pad8(out[3]), GZT[3], ldt, loss_dev);
-    e = cudaGetLastError();
+// Loss and gradient of one batch into loss_dev and grad: the input rows, four forward
+// layers (the last with the loss), three backward layers, the weight gradients and the sums.
+int Mlp::loss_gradient(const float* lnT, const float* b1, const float* target, int B, cudaStream_t st) {
+  mlp_input_kernel<<<blocks_for(B), 256, 0, st>>>(lnT, b1, B, norm[0], norm[1], norm[2], norm[3], norm[4], norm[5],
+                                                  X[0]);
+  cudaError_t e = cudaGetLastError();
+  LayerIo io;
+  io.scale = scale_dev;
+  io.target = target;
+  io.lam = lam;
+  io.losspart = losspart;
+  io.lnT = lnT;
+  io.b1 = b1;
+  for (int k = 0; k < 6; ++k) io.norm[k] = norm[k];
+  for (int l = 0; l < 4 && e == cudaSuccess; ++l) {
+    io.bias = theta + off[l] + (int64_t)out[l] * in[l];
+    io.za = ZA[l];
+    io.xn = l < 3 ? X[l + 1] : GZ[3];
+    io.ldn = l < 3 ? pad8(in[l + 1]) : pad8(out[3]);
+    io.colpart = colpart[l];
+    e = l < 3 ? launch_layer<kTrainHidden>(xmap[l], wmap64[l], B, out[l], in[l], io, sms, dev_err, st)
+              : launch_layer<kTrainLast>(xmap[l], wmap64[l], B, out[l], in[l], io, sms, dev_err, st);
   }
-  if (e == cudaSuccess) {
-    mlp_out_bias_grad_kernel<<<R, 256, 0, st>>>(Z[3], b4, scale_dev, target, B, R,
-                                                grad + off[3] + (int64_t)out[3] * in[3]);
-    e = cudaGetLastError();
-  }
-  for (int l = 3; l >= 0 && e == cudaSuccess; --l) {
-    // dW_l = GZ_l^T X_l over all 3B rows
-    e = launch_tc_gemm(opGZT[l], opXT[l], grad + off[l], out[l], in[l], Mc, in[l], 1, nullptr, dev_err, st);
-    if (e != cudaSuccess || l == 0) break;
-    // dL/dX_l = GZ_l W_l, then back through layer l-1's tanh
-    e = launch_tc_gemm(opGZ[l], opWT[l], GX, Mc, in[l], out[l], in[l], 1, nullptr, dev_err, st);
-    if (e != cudaSuccess) break;
+  // dL/dX_l = GZ_l W_l, then back through layer l - 1's tanh.  dW_3 and dW_2 run on streams
+  // of their own as soon as their gradient rows stand, dW_1 on the caller's beside the last
+  // backward layer (side 2); everything is joined below.
+  auto dw = [&](int l, cudaStream_t s) {
+    const int tiles = ((out[l] + tc::BM - 1) / tc::BM) * (in[l] / kDwN);
+    mlp_dw_kernel<<<tiles, 128, kDwSmem, s>>>(gzmap_k[l], xmap_k[l], 3 * B, out[l], in[l], grad + off[l], dev_err);
+    return cudaGetLastError();
+  };
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(mlp_dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDwSmem);
+  int forked = 0;  // side streams with work on them
+  auto fork = [&](int k) {
+    cudaError_t r = cudaEventRecord(ev_fork[k], st);
+    if (r == cudaSuccess) r = cudaStreamWaitEvent(side[k], ev_fork[k], 0);
+    if (r == cudaSuccess) forked = k + 1;
+    return r;
+  };
+  for (int l = 3; l > 0 && e == cudaSuccess; --l) {
     const int lp = l - 1;
-    mlp_backact_kernel<<<blocks_for((int64_t)B * out[lp]), 256, 0, st>>>(
-        GX, Z[lp], theta + off[lp] + (int64_t)out[lp] * in[lp], B, out[lp], GZ[lp], pad8(out[lp]), GZT[lp], ldt,
-        grad + off[lp] + (int64_t)out[lp] * in[lp]);
-    e = cudaGetLastError();
+    io.za = ZA[lp];
+    io.xn = GZ[lp];  // not kept for layer 0
+    io.ldn = pad8(out[lp]);
+    io.colpart = colpart[lp];
+    e = fork(3 - l);
+    if (e != cudaSuccess) break;
+    if (lp > 0) {
+      e = dw(l, side[3 - l]);
+      if (e == cudaSuccess)
+        e = launch_layer<kBack>(gzmap[l], wtmap64[l], B, in[l], out[l], io, sms, dev_err, st);
+    } else {
+      e = launch_layer<kBackFirst>(gzmap[l], wtmap64[l], B, in[l], out[l], io, sms, dev_err, side[2]);
+      if (e == cudaSuccess) {
+        // layer 0's tangent inputs as the GEMM operand holds them
+        const float d1 = host_bf16_to_float(host_bf16(1.f / norm[1]));
+        const float d2 = host_bf16_to_float(host_bf16(1.f / norm[3]));
+        const int prows = 4 * ((B + tc::BM - 1) / tc::BM);
+        e = launch_pdl(mlp_grad_sum_kernel, dim3((3 * H + R + 31) / 32 + 1), dim3(32 * kSumWarps), 0, side[2],
+                       colpart[0], colpart[1], colpart[2], colpart[3], losspart, prows * ((R + 7) / 8), prows, H, R, B,
+                       d1, d2, grad, loss_dev);
+      }
+      if (e == cudaSuccess) e = dw(1, st);
+    }
   }
-  return e == cudaSuccess ? MRSTAT_OK : cuda_fail(e, "surrogate backward");
+  // join, also after an error: the caller's stream owns the buffers
+  for (int k = 0; k < forked; ++k) {
+    cudaError_t r = cudaEventRecord(ev_join[k], side[k]);
+    if (r == cudaSuccess) r = cudaStreamWaitEvent(st, ev_join[k], 0);
+    if (e == cudaSuccess) e = r;
+  }
+  return e == cudaSuccess ? MRSTAT_OK : cuda_fail(e, "surrogate gradient");
 }
 
 int Mlp::adam(float lr, cudaStream_t st) {
@@ -683,24 +981,6 @@ int Mlp::adam(float lr, cudaStream_t st) {
 }
 
 
-template <bool LAST>
-static cudaError_t launch_persistent(const TcOperand& x, const CUtensorMap& w64, int B, int N, int K,
-                                     const float* bias, __nv_bfloat16* xn, int ldn, const float* scale, float* pred,
-                                     int* err, cudaStream_t st) {
-  const size_t sm = PerShape::kSmem;
-  cudaError_t e = cudaFuncSetAttribute(mlp_layer_persistent_kernel<LAST>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0;
-  e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess) return e;
-  const int tiles = ((B + tc::BM - 1) / tc::BM) * ((N + PerShape::BN - 1) / PerShape::BN);
-  const int grid = std::max(1, std::min(tiles, sms));
-  mlp_layer_persistent_kernel<LAST><<<grid, kPerThreads, sm, st>>>(x.hi, w64, B, N, K, bias, xn, ldn, scale, pred, err);
-  return cudaGetLastError();
-}
-
 // Inference: layer 0 on the CUDA cores, then one persistent fused tensor-core kernel per
 // layer (no pre-activation buffers).
 int Mlp::infer_fused(const float* lnT, const float* b1, int B, float* pred, cudaStream_t st) {
@@ -711,14 +991,15 @@ int Mlp::infer_fused(const float* lnT, const float* b1, int B, float* pred, cuda
         theta + off[0] + (int64_t)out[0] * in[0], out[0], X[1], pad8(in[1]));
   }
   cudaError_t e = cudaGetLastError();
+  LayerIo io;
+  io.scale = scale_dev;
+  io.pred = pred;
   for (int l = 1; l < 4 && e == cudaSuccess; ++l) {
-    const float* bias = theta + off[l] + (int64_t)out[l] * in[l];
-    const bool last = l == 3;
-    __nv_bfloat16* xn = last ? nullptr : X[l + 1];
-    const int ldn = last ? 0 : pad8(in[l + 1]);
-    e = last ? launch_persistent<true>(opX[l], wmap64[l], B, out[l], in[l], bias, xn, ldn, scale_dev, pred, dev_err, st)
-             : launch_persistent<false>(opX[l], wmap64[l], B, out[l], in[l], bias, xn, ldn, scale_dev, pred, dev_err,
-                                        st);
+    io.bias = theta + off[l] + (int64_t)out[l] * in[l];
+    io.xn = l < 3 ? X[l + 1] : nullptr;
+    io.ldn = l < 3 ? pad8(in[l + 1]) : 0;
+    e = l < 3 ? launch_layer<kInferHidden>(xmap[l], wmap64[l], B, out[l], in[l], io, sms, dev_err, st)
+              : launch_layer<kInferLast>(xmap[l], wmap64[l], B, out[l], in[l], io, sms, dev_err, st);
   }
   return e == cudaSuccess ? MRSTAT_OK : cuda_fail(e, "surrogate inference");
 }
@@ -815,8 +1096,7 @@ int mrstat_mlp_train_step(mrstat_mlp* m, const float* lnT, const float* b1, cons
   DeviceGuard g(m->device);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   int s = m->ensure_batch(B, true);
-  if (s == MRSTAT_OK) s = m->forward(lnT, b1, B, true, st);
-  if (s == MRSTAT_OK) s = m->backward(target, B, st);
+  if (s == MRSTAT_OK) s = m->loss_gradient(lnT, b1, target, B, st);
   if (s == MRSTAT_OK && lr > 0) s = m->adam(lr, st);
   if (s == MRSTAT_OK && loss_out != nullptr) {
     cudaError_t e = cudaMemcpyAsync(loss_out, m->loss_dev, sizeof(double), cudaMemcpyDeviceToDevice, st);
@@ -833,16 +1113,17 @@ int mrstat_mlp_loss_grad(mrstat_mlp* m, const float* lnT, const float* b1, const
   DeviceGuard g(m->device);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   int s = m->ensure_batch(B, true);
-  if (s == MRSTAT_OK) s = m->forward(lnT, b1, B, true, st);
-  if (s == MRSTAT_OK) s = m->backward(target, B, st);
+  if (s == MRSTAT_OK) s = m->loss_gradient(lnT, b1, target, B, st);
   if (s != MRSTAT_OK) return s;
   cudaError_t e = cudaSuccess;
   if (grad) e = cudaMemcpyAsync(grad, m->grad, m->np * sizeof(float), cudaMemcpyDeviceToDevice, st);
-  if (e == cudaSuccess && loss_host) e = cudaMemcpyAsync(loss_host, m->loss_dev, sizeof(double), cudaMemcpyDeviceToHost, st);
+  // the loss and the error flag in one copy and one wait
+  if (e == cudaSuccess) e = cudaMemcpyAsync(m->stat_host, m->stat, 2 * sizeof(double), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  int herr = 0;
-  if (e == cudaSuccess) e = cudaMemcpy(&herr, m->dev_err, sizeof(int), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(e, "surrogate gradient");
+  if (loss_host) *loss_host = m->stat_host[0];
+  int herr = 0;
+  std::memcpy(&herr, m->stat_host + 1, sizeof(int));
   if (herr) {
     cudaMemset(m->dev_err, 0, sizeof(int));
     return fail(MRSTAT_ERR_TIMEOUT, "a tensor-core kernel gave up waiting on its pipeline barriers");

@@ -23,27 +23,29 @@ struct Mlp {
   std::vector<float> scale_host;
   __nv_bfloat16* Wb[4] = {nullptr, nullptr, nullptr, nullptr};   // bf16 [out][pad8(in)]
   __nv_bfloat16* WTb[4] = {nullptr, nullptr, nullptr, nullptr};  // bf16 [in][pad8(out)]
-  TcOperand opW[4], opWT[4];
-  CUtensorMap wmap64[4];  // the weights with 64-row boxes (the persistent inference layers)
+  CUtensorMap wmap64[4], wtmap64[4];  // the weights and their transposes, 64-row boxes
   // batch buffers (M = 3 B rows: values, ln T1 tangents, ln T2 tangents)
-  int cap = 0, maps_b = -1;
+  int cap = 0, maps_b = -1, sms = 1;
   bool maps_train = false, have_train_buffers = false;
   __nv_bfloat16* X[4] = {nullptr, nullptr, nullptr, nullptr};    // bf16 [M][pad8(in)] layer inputs
-  __nv_bfloat16* XT[4] = {nullptr, nullptr, nullptr, nullptr};   // bf16 [in][pad8(3 cap)]
-  float* Z[4] = {nullptr, nullptr, nullptr, nullptr};   // [M][out] pre-activations (no bias; training)
-  __nv_bfloat16* GZ[4] = {nullptr, nullptr, nullptr, nullptr};   // bf16 [M][pad8(out)]
-  __nv_bfloat16* GZT[4] = {nullptr, nullptr, nullptr, nullptr};  // bf16 [out][pad8(3 cap)]
-  float* GX = nullptr;                                  // [M][H]
+  float* ZA[4] = {nullptr, nullptr, nullptr, nullptr};           // [3][B][out] a, z1, z2 of layers 0..2 (training)
+  __nv_bfloat16* GZ[4] = {nullptr, nullptr, nullptr, nullptr};   // bf16 [M][pad8(out)] gradient rows, layers 1..3
+  float* colpart[4] = {nullptr, nullptr, nullptr, nullptr};      // column sums of the row tiles (biases, layer 0)
+  double* losspart = nullptr;
+  CUtensorMap xmap[4], gzmap[4];      // 128-row boxes, columns as the GEMM's K
+  CUtensorMap xmap_k[4], gzmap_k[4];  // 64-row boxes, rows as the GEMM's K
+  double* stat = nullptr;             // device: the loss, then the error flag of a bounded wait
+  double* stat_host = nullptr;        // its pinned copy
+  cudaStream_t side[3] = {nullptr, nullptr, nullptr};  // a gradient's independent launches
+  cudaEvent_t ev_fork[3] = {nullptr, nullptr, nullptr}, ev_join[3] = {nullptr, nullptr, nullptr};
   double* loss_dev = nullptr;
-  TcOperand opX[4], opXT[4], opGZ[4], opGZT[4];
   int* dev_err = nullptr;
 
   ~Mlp();
   int setup(int h, int r, uint64_t seed);
   int set_params(const float* host, cudaStream_t st);
   int ensure_batch(int B, bool train);
-  int forward(const float* lnT, const float* b1, int B, bool train, cudaStream_t st);
-  int backward(const float* target, int B, cudaStream_t st);
+  int loss_gradient(const float* lnT, const float* b1, const float* target, int B, cudaStream_t st);
   int adam(float lr, cudaStream_t st);
   int infer_fused(const float* lnT, const float* b1, int B, float* pred, cudaStream_t st);
   void release_batch();

@@ -114,7 +114,23 @@ __device__ __forceinline__ uint64_t sdesc_sw128(const void* tile) {
   return d;
 }
 
-// Instruction descriptor of kind::f16: F32 accumulator, BF16 A and B, both K-major.
+// MN-major operand, 128-byte swizzle: tiles of 64 MN elements (128 B) by K rows; blocks of 64
+// MN elements are mn_stride bytes apart (leading byte offset), groups of 8 K rows 1024 B
+// (stride byte offset), so a K step of 16 rows advances the start address by 2048 B.
+__device__ __forceinline__ uint64_t sdesc_sw128_mn(const void* tile, uint32_t mn_stride) {
+  const uint64_t a = smem_u32(tile);
+  uint64_t d = (a >> 4) & 0x3FFFull;
+  d |= (uint64_t)(mn_stride >> 4) << 16;
+  d |= (uint64_t)(1024 >> 4) << 32;
+  d |= 1ull << 46;
+  d |= 2ull << 61;
+  return d;
+}
+
+constexpr uint32_t kIdescMnMajorA = 1u << 15, kIdescMnMajorB = 1u << 16;
+
+// Instruction descriptor of kind::f16: F32 accumulator, BF16 A and B, both K-major (or
+// MN-major with the flags above).
 __host__ __device__ constexpr uint32_t make_idesc(int m, int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
@@ -146,6 +162,16 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 }  // namespace tc
