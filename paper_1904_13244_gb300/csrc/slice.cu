@@ -11,165 +11,213 @@
 //   mean of m_y over the isochromats (the x components cancel by the slice's mirror
 //   symmetry, so the signal stays i * mean m_y).
 //
-// One lane per isochromat (n_iso a power of two <= 32, 32 / n_iso voxels per warp), the
-// whole 3-vector state and its ln T1 / ln T2 tangents in registers.  The pulse of a
-// (TR, isochromat) pair does not depend on the voxel: mrstat_set_slice_profile composes
-// each one once, in float64 on the host, into a 3 x 3 matrix (columns: the basis vectors
-// pushed through pre-winder, sub-steps and rewinder); each block stages a chunk of TRs'
-// matrices in shared memory and its lanes apply them; the per-voxel sum over the
-// isochromats is a segmented shuffle reduction, written as TR quads like K1.
+// Mirror symmetry halves the isochromats: u_k = -u_{n_iso-1-k}, so the two see opposite
+// precessions, and (m_x, m_y, m_z) -> (-m_x, m_y, m_z) maps one recursion to the other; the
+// mean of m_y runs over k < n_iso / 2.  A lane carries two of them in packed float32 pairs
+// (packed.cuh): 8 lanes per voxel for 32 isochromats, 4 voxels per warp, the 3-vector state
+// and its ln T1 / ln T2 tangents in registers.  The relaxation over TE and over TR - TE act
+// on the same state one after the other, so the state takes both as one step over TR; the
+// echo, which only the first step reaches, is E2(TE) times the sum over the isochromats
+// (plus its ln T2 source), applied once per voxel after the sum.  The pulse of a (TR,
+// isochromat) pair does not depend on the voxel: mrstat_set_slice_profile composes each one
+// once, in float64 on the host, into a 3 x 3 matrix (columns: the basis vectors pushed
+// through pre-winder, sub-steps and rewinder); each block stages a chunk of TRs' matrices in
+// shared memory and its lanes apply them.
+//
+// Bound by the FP32 pipe: per TR and isochromat pair 27 packed multiply-adds for the pulse
+// on the state and both tangents and 13 for the relaxation.  At 224 x 224, 1120 TRs and 32
+// isochromats: 1.63 ms with the tangents, 0.59 ms for m alone (5.86 and 5.61 ms with one
+// lane per isochromat and the two decays).
+#include <algorithm>
+#include <cmath>
+
 #include "internal.cuh"
+#include "packed.cuh"
 
 namespace mrstat {
 namespace {
 
-constexpr int kSliceThreads = 512;
-constexpr int kSliceChunk = 16;  // TRs per composed chunk: kSliceChunk * n_iso <= kSliceThreads
+constexpr int kSliceThreads = 256;
+constexpr int kSliceChunk = 16;  // TRs per staged chunk
 constexpr int kSliceMaxSub = 64;
+constexpr int kRotStride = 10;   // pairs per (TR, isochromat pair): 9 and padding to 16 bytes
 
+// L lanes per voxel group (L = 1, 2, 4, 8 isochromat pairs), V voxels per lane sharing each
+// loaded matrix; NCH 1: m only, 3: with both tangents.
+template <int L, int NCH, int V>
 __global__ void __launch_bounds__(kSliceThreads)
 bloch_slice_kernel(const float* __restrict__ alpha, const uint8_t* __restrict__ mask,
-                   const float* __restrict__ rotg, int n_iso, int log2_iso, int nv, int nq, float te, float tb,
-                   float m0z, int nch, float4* __restrict__ D) {
-  __shared__ float rot[kSliceChunk * 32 * 9];  // [TR in chunk][isochromat][3 x 3, column-major]
+                   const float2* __restrict__ rotg, int nv, int nq, float te, float tr, float m0z,
+                   float4* __restrict__ D) {
+  using pk::f2;
+  constexpr int kVals = 4 * NCH;              // echo values of a TR quad
+  constexpr int kHalves = L < 4 ? L : 4;      // lanes that share them after the exchanges
+  constexpr int kKeep = kVals / kHalves;      // values a lane ends with: 4 / kHalves TRs
+  __shared__ __align__(16) f2 rot[kSliceChunk * L * kRotStride];
   const int tid = threadIdx.x, lane = tid & 31;
-  const int k = lane & (n_iso - 1);                              // this lane's isochromat
-  const int j = ((blockIdx.x * kSliceThreads + tid) >> 5) * (32 >> log2_iso) + (lane >> log2_iso);
-  const bool live = j < nv;
-  const bool on = live && (mask == nullptr || mask[j] != 0);
+  const int p = lane & (L - 1);  // this lane's isochromat pair
+  const int j0 = ((blockIdx.x * kSliceThreads + tid) >> 5) * (V * 32 / L) + lane / L;
   const size_t cstride = (size_t)nq * nv;
 
-  float t1 = 1000.f, t2 = 100.f;
-  if (live) {
-    t1 = expf(alpha[j]);
-    t2 = expf(alpha[nv + j]);
+  // over TR: m += (E - 1)(m - m_eq) with E - 1 from expm1f; d = dE/dln T.  Over TE the
+  // transverse factor and its derivative, for the echo
+  const f2 minus1 = pk::both(-1.f), zero = pk::both(0.f);
+  f2 x1[V], x2[V], d1[V], d2[V], m[V][3], a[V][3], b[V][3];
+  float x2e[V], d2e[V], norm[V];
+  bool any = false;
+#pragma unroll
+  for (int w = 0; w < V; ++w) {
+    const int j = j0 + w * (32 / L);
+    const bool live = j < nv;
+    const bool on = live && (mask == nullptr || mask[j] != 0);
+    any |= on;
+    float t1 = 1000.f, t2 = 100.f;
+    if (live) {
+      t1 = expf(alpha[j]);
+      t2 = expf(alpha[nv + j]);
+    }
+    const float x1s = expm1f(-tr / t1), x2s = expm1f(-tr / t2);
+    x1[w] = pk::both(x1s);
+    x2[w] = pk::both(x2s);
+    d1[w] = pk::both(tr / t1 * (1.f + x1s));
+    d2[w] = pk::both(tr / t2 * (1.f + x2s));
+    x2e[w] = expm1f(-te / t2);
+    d2e[w] = te / t2 * (1.f + x2e[w]);
+    norm[w] = on ? 1.f / (float)(2 * L) : 0.f;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) m[w][i] = a[w][i] = b[w][i] = zero;
+    m[w][2] = pk::both(m0z);
   }
-  // decay factors as in K1: m += (E - 1)(m - m_eq) with E - 1 from expm1f; d = dE/dln T
-  const float ra1 = te / t1, ra2 = te / t2, rb1 = tb / t1, rb2 = tb / t2;
-  const float x1a = expm1f(-ra1), x2a = expm1f(-ra2), x1b = expm1f(-rb1), x2b = expm1f(-rb2);
-  const float d1a = ra1 * (1.f + x1a), d2a = ra2 * (1.f + x2a);
-  const float d1b = rb1 * (1.f + x1b), d2b = rb2 * (1.f + x2b);
+  const bool work = __any_sync(0xffffffffu, any);  // a warp outside the mask only writes zeros
 
-  float m[3] = {0.f, 0.f, m0z}, a[3] = {0.f, 0.f, 0.f}, b[3] = {0.f, 0.f, 0.f};
-  float o0[4], o1[4], o2[4];
-  const float inv_iso = 1.f / (float)n_iso;
   const int ntr4 = 4 * nq;
-
   for (int n0 = 0; n0 < ntr4; n0 += kSliceChunk) {
     __syncthreads();  // the previous chunk's matrices are no longer read
-    // the chunk's composed pulses (TRs past the train are never applied)
-    const int nrot = min(kSliceChunk, ntr4 - n0) * 32 * 9;
-    const float* src = rotg + (size_t)n0 * 32 * 9;
-    for (int e = tid; e < nrot; e += kSliceThreads) rot[e] = __ldg(src + e);
+    const int cnt = min(kSliceChunk, ntr4 - n0);
+    {
+      const float4* src = reinterpret_cast<const float4*>(rotg + (size_t)n0 * L * kRotStride);
+      float4* dst = reinterpret_cast<float4*>(rot);
+      for (int e = tid; e < cnt * L * kRotStride / 2; e += kSliceThreads) dst[e] = __ldg(src + e);
+    }
     __syncthreads();
-    for (int nq4 = 0; nq4 < kSliceChunk; nq4 += 4) {
-      if (n0 + nq4 >= ntr4) break;  // ntr4 and the quads are multiples of 4
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int nn = nq4 + u;
-        const float* R = rot + (nn * 32 + k) * 9;  // columns R[0..2], R[3..5], R[6..8]
-        float r[9];
-#pragma unroll
-        for (int e = 0; e < 9; ++e) r[e] = R[e];
-        float v[3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) v[i] = fmaf(r[i], m[0], fmaf(r[3 + i], m[1], r[6 + i] * m[2]));
-        m[0] = v[0], m[1] = v[1], m[2] = v[2];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) v[i] = fmaf(r[i], a[0], fmaf(r[3 + i], a[1], r[6 + i] * a[2]));
-        a[0] = v[0], a[1] = v[1], a[2] = v[2];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) v[i] = fmaf(r[i], b[0], fmaf(r[3 + i], b[1], r[6 + i] * b[2]));
-        b[0] = v[0], b[1] = v[1], b[2] = v[2];
-        // decay over TE with the tangents' source terms (taken from the state before decay)
-        float zm1 = m[2] - 1.f;
-        a[0] = fmaf(x2a, a[0], a[0]);
-        a[1] = fmaf(x2a, a[1], a[1]);
-        a[2] = fmaf(x1a, a[2], fmaf(d1a, zm1, a[2]));
-        b[0] = fmaf(x2a, b[0], fmaf(d2a, m[0], b[0]));
-        b[1] = fmaf(x2a, b[1], fmaf(d2a, m[1], b[1]));
-        b[2] = fmaf(x1a, b[2], b[2]);
-        m[0] = fmaf(x2a, m[0], m[0]);
-        m[1] = fmaf(x2a, m[1], m[1]);
-        m[2] = fmaf(x1a, zm1, m[2]);
-        // echo: the mean of m_y (and tangents) over the voxel's isochromats; with 32
-        // isochromats (one voxel per warp) the quad's twelve sums are formed together after
-        // the quad, otherwise per TR here
-        if (n_iso == 32) {
-          o0[u] = m[1];
-          o1[u] = a[1];
-          o2[u] = b[1];
-        } else {
-          float sy = m[1], sa = a[1], sb = b[1];
-          for (int o = n_iso >> 1; o > 0; o >>= 1) {
-            sy += __shfl_xor_sync(0xffffffffu, sy, o);
-            sa += __shfl_xor_sync(0xffffffffu, sa, o);
-            sb += __shfl_xor_sync(0xffffffffu, sb, o);
-          }
-          o0[u] = sy * inv_iso;
-          o1[u] = sa * inv_iso;
-          o2[u] = sb * inv_iso;
-        }
-        // decay over TR - TE
-        zm1 = m[2] - 1.f;
-        a[0] = fmaf(x2b, a[0], a[0]);
-        a[1] = fmaf(x2b, a[1], a[1]);
-        a[2] = fmaf(x1b, a[2], fmaf(d1b, zm1, a[2]));
-        b[0] = fmaf(x2b, b[0], fmaf(d2b, m[0], b[0]));
-        b[1] = fmaf(x2b, b[1], fmaf(d2b, m[1], b[1]));
-        b[2] = fmaf(x1b, b[2], b[2]);
-        m[0] = fmaf(x2b, m[0], m[0]);
-        m[1] = fmaf(x2b, m[1], m[1]);
-        m[2] = fmaf(x1b, zm1, m[2]);
-      }
-      if (n_iso == 32) {
-        // the quad's twelve sums v[3 u + channel] over the warp's lanes, by halving: after
-        // the exchanges across lane bits 4 and 3, lane group g = lane / 8 holds TR u = g's
-        // three values, summed over its partners; a butterfly over the low three lane bits
-        // completes them (18 shuffles for the quad instead of 60)
-        float v[12];
+    for (int nq4 = 0; nq4 < cnt; nq4 += 4) {  // ntr4 and the quads are multiples of 4
+      float v[V][kVals];
+      if (work) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          v[3 * u] = o0[u];
-          v[3 * u + 1] = o1[u];
-          v[3 * u + 2] = o2[u];
-        }
-        const bool h4 = (lane & 16) != 0, h3 = (lane & 8) != 0;
-        float w[6], x[3];
+          const ulonglong2* R2 = reinterpret_cast<const ulonglong2*>(rot + ((nq4 + u) * L + p) * kRotStride);
+          f2 r[10];  // columns r[0..2], r[3..5], r[6..8]
 #pragma unroll
-        for (int e = 0; e < 6; ++e) {
-          const float send = h4 ? v[e] : v[6 + e], keep = h4 ? v[6 + e] : v[e];
-          w[e] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-        }
+          for (int e = 0; e < 5; ++e) {
+            const ulonglong2 t = R2[e];
+            r[2 * e] = t.x;
+            r[2 * e + 1] = t.y;
+          }
+          auto turn = [&](f2 (&s)[3]) {
+            f2 w[3];
 #pragma unroll
-        for (int e = 0; e < 3; ++e) {
-          const float send = h3 ? w[e] : w[3 + e], keep = h3 ? w[3 + e] : w[e];
-          x[e] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-        }
+            for (int i = 0; i < 3; ++i) w[i] = pk::fma(r[i], s[0], pk::fma(r[3 + i], s[1], pk::mul(r[6 + i], s[2])));
+            s[0] = w[0], s[1] = w[1], s[2] = w[2];
+          };
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1)
-#pragma unroll
-          for (int e = 0; e < 3; ++e) x[e] += __shfl_xor_sync(0xffffffffu, x[e], o);
-        if ((lane & 7) == 0 && live) {  // TR u of the quad: one float of each channel's float4
-          const int u = lane >> 3;
-          const size_t q = (size_t)((n0 + nq4) >> 2) * nv + j;
-          __stcs(reinterpret_cast<float*>(D + q) + u, on ? x[0] * inv_iso : 0.f);
-          if (nch > 1) {
-            __stcs(reinterpret_cast<float*>(D + cstride + q) + u, on ? x[1] * inv_iso : 0.f);
-            __stcs(reinterpret_cast<float*>(D + 2 * cstride + q) + u, on ? x[2] * inv_iso : 0.f);
+          for (int w = 0; w < V; ++w) {
+            turn(m[w]);
+            const float2 my = pk::split(m[w][1]);
+            v[w][NCH * u] = my.x + my.y;
+            if (NCH > 1) {
+              turn(a[w]);
+              turn(b[w]);
+              const float2 ay = pk::split(a[w][1]), by = pk::split(b[w][1]);
+              v[w][NCH * u + 1] = ay.x + ay.y;
+              v[w][NCH * u + 2] = by.x + by.y;
+            }
+            // decay over TR with the tangents' source terms (from the state before it)
+            const f2 zm1 = pk::add(m[w][2], minus1);
+            if (NCH > 1) {
+              a[w][0] = pk::fma(x2[w], a[w][0], a[w][0]);
+              a[w][1] = pk::fma(x2[w], a[w][1], a[w][1]);
+              a[w][2] = pk::fma(x1[w], a[w][2], pk::fma(d1[w], zm1, a[w][2]));
+              b[w][0] = pk::fma(x2[w], b[w][0], pk::fma(d2[w], m[w][0], b[w][0]));
+              b[w][1] = pk::fma(x2[w], b[w][1], pk::fma(d2[w], m[w][1], b[w][1]));
+              b[w][2] = pk::fma(x1[w], b[w][2], b[w][2]);
+            }
+            m[w][0] = pk::fma(x2[w], m[w][0], m[w][0]);
+            m[w][1] = pk::fma(x2[w], m[w][1], m[w][1]);
+            m[w][2] = pk::fma(x1[w], zm1, m[w][2]);
           }
         }
-      } else if (k == 0 && live) {  // one float4 per channel and TR quad, as K1 stores them
+        // the quad's sums over the voxel's L lanes by halving: each exchange leaves a lane
+        // with the half of the TRs its lane bit names; for L = 8 the lowest bit is added last
+        if constexpr (L >= 2) {
+#pragma unroll
+          for (int w = 0; w < V; ++w) {
+#pragma unroll
+            for (int off = L / 2, n = kVals; n > kKeep; off >>= 1, n >>= 1) {
+              const bool up = lane & off;
+#pragma unroll
+              for (int e = 0; e < n / 2; ++e) {
+                const float send = up ? v[w][e] : v[w][n / 2 + e], keep = up ? v[w][n / 2 + e] : v[w][e];
+                v[w][e] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+              }
+            }
+            if constexpr (L == 8) {
+#pragma unroll
+              for (int e = 0; e < kKeep; ++e) v[w][e] += __shfl_xor_sync(0xffffffffu, v[w][e], 1);
+            }
+          }
+        }
+      } else {
+#pragma unroll
+        for (int w = 0; w < V; ++w)
+#pragma unroll
+          for (int e = 0; e < kKeep; ++e) v[w][e] = 0.f;
+      }
+      if (L == 8 && (lane & 1)) continue;
+      const int u0 = (L == 8 ? p >> 1 : p) * (4 / kHalves);  // this lane's first TR of the quad
+#pragma unroll
+      for (int w = 0; w < V; ++w) {
+        const int j = j0 + w * (32 / L);
+        if (j >= nv) continue;
         const size_t q = (size_t)((n0 + nq4) >> 2) * nv + j;
-        const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-        __stcs(D + q, on ? make_float4(o0[0], o0[1], o0[2], o0[3]) : z4);
-        if (nch > 1) {  // the tangent channels (absent from the forward-only buffer)
-          __stcs(D + cstride + q, on ? make_float4(o1[0], o1[1], o1[2], o1[3]) : z4);
-          __stcs(D + 2 * cstride + q, on ? make_float4(o2[0], o2[1], o2[2], o2[3]) : z4);
+#pragma unroll
+        for (int t = 0; t < 4 / kHalves; ++t) {
+          const float sm = v[w][NCH * t] * norm[w];
+          __stcs(reinterpret_cast<float*>(D + q) + u0 + t, fmaf(x2e[w], sm, sm));
+          if (NCH > 1) {
+            const float sa = v[w][NCH * t + 1] * norm[w], sb = v[w][NCH * t + 2] * norm[w];
+            __stcs(reinterpret_cast<float*>(D + cstride + q) + u0 + t, fmaf(x2e[w], sa, sa));
+            __stcs(reinterpret_cast<float*>(D + 2 * cstride + q) + u0 + t, fmaf(x2e[w], sb, fmaf(d2e[w], sm, sb)));
+          }
         }
       }
     }
   }
+}
+
+// Isochromat pairs per voxel (lanes): the first half of the isochromats, two per lane; one
+// or two isochromats fill one lane's pair with the same isochromat twice.
+int slice_pairs(int n_iso) { return n_iso >= 4 ? n_iso / 4 : 1; }
+
+template <int L, int NCH, int V>
+cudaError_t launch_slice_t(const Plan& p, const float* alpha, const uint8_t* mask, float4* D, cudaStream_t st) {
+  const int vpb = kSliceThreads / L * V;  // voxels per block
+  bloch_slice_kernel<L, NCH, V><<<(p.nv + vpb - 1) / vpb, kSliceThreads, 0, st>>>(
+      alpha, mask, reinterpret_cast<const float2*>(p.slice_rot), p.nv, p.nq, (float)p.te_ms, (float)p.tr_ms,
+      p.inversion ? -1.f : 1.f, D);
+  return cudaGetLastError();
+}
+
+// Without the tangents four voxels per lane share each loaded matrix (the shared-memory
+// reads, five 16-byte loads per TR and lane, are then what one voxel per lane is bound by:
+// 1.02 against 0.59 ms at 224 x 224, 1120 TRs, 32 isochromats), where that still leaves the
+// SMs two warps per scheduler; with them the FP32 pipe is, and one voxel per lane keeps more
+// warps in flight (1.63 against 1.75 ms with two).
+template <int L>
+cudaError_t launch_slice(const Plan& p, const float* alpha, const uint8_t* mask, float4* D, int nch, cudaStream_t st) {
+  if (nch > 1) return launch_slice_t<L, 3, 1>(p, alpha, mask, D, st);
+  const int64_t warps = ((int64_t)p.nv * L + 31) / 32;
+  return warps >= 4 * 8 * 152 ? launch_slice_t<L, 1, 4>(p, alpha, mask, D, st)
+                              : launch_slice_t<L, 1, 1>(p, alpha, mask, D, st);
 }
 
 }  // namespace
@@ -177,14 +225,12 @@ bloch_slice_kernel(const float* __restrict__ alpha, const uint8_t* __restrict__ 
 cudaError_t launch_bloch_slice(const Plan& p, const float* alpha, const uint8_t* mask, float4* D, int nch,
                                cudaStream_t st) {
   if (p.nv == 0) return cudaSuccess;
-  const int vpb = (kSliceThreads / 32) * (32 / p.slice_iso);  // voxels per block
-  const int blocks = (p.nv + vpb - 1) / vpb;
-  const float te = (float)p.te_ms, tb = (float)(p.tr_ms - p.te_ms);
-  int log2_iso = 0;
-  while ((1 << log2_iso) < p.slice_iso) ++log2_iso;
-  bloch_slice_kernel<<<blocks, kSliceThreads, 0, st>>>(alpha, mask, p.slice_rot, p.slice_iso, log2_iso, p.nv,
-                                                      p.nq, te, tb, p.inversion ? -1.f : 1.f, nch, D);
-  return cudaGetLastError();
+  switch (slice_pairs(p.slice_iso)) {
+    case 1: return launch_slice<1>(p, alpha, mask, D, nch, st);
+    case 2: return launch_slice<2>(p, alpha, mask, D, nch, st);
+    case 4: return launch_slice<4>(p, alpha, mask, D, nch, st);
+    default: return launch_slice<8>(p, alpha, mask, D, nch, st);
+  }
 }
 
 }  // namespace mrstat
@@ -218,16 +264,20 @@ int mrstat_set_slice_profile(mrstat_plan* plan, const mrstat_slice_profile* prof
     sum += w[s];
   }
   cudaError_t e = cudaSuccess;
-  if (p->slice_rot == nullptr) e = dalloc(p, &p->slice_rot, (size_t)p->ntr_pad * 32 * 9);
+  constexpr size_t kMaxPairs = 8;
+  if (p->slice_rot == nullptr) e = dalloc(p, &p->slice_rot, (size_t)p->ntr_pad * kMaxPairs * kRotStride * 2);
   // the composed pulse of every (TR, isochromat): pre-winder, then per sub-step the RF
   // rotation by phi_n w_s about the TR's axis (the hard-pulse kernel's convention) and the
   // precession by beta_k, then the rewinder; in float64 from the plan's signed flips
   std::vector<float> phi(p->ntr_pad);
   if (e == cudaSuccess) e = cudaMemcpy(phi.data(), p->phi, phi.size() * sizeof(float), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(e, "slice profile tables");
-  std::vector<float> rot((size_t)p->ntr_pad * 32 * 9, 0.f);
+  // for the isochromats of the first half, laid out as pairs [TR][pair][9 + padding][2]
+  const int pairs = slice_pairs(ni), half_iso = ni > 1 ? ni / 2 : 1;
+  std::vector<float> rot((size_t)p->ntr_pad * pairs * kRotStride * 2, 0.f);
   for (int n = 0; n < p->ntr_pad; ++n)
-    for (int k = 0; k < ni; ++k) {
+    for (int kk = 0; kk < 2 * pairs; ++kk) {
+      const int k = std::min(kk, half_iso - 1);
       const double u = prof->extent * ((k + 0.5) / ni - 0.5);
       const double beta = 2.0 * M_PI * prof->tbw * u / ns, half = -0.5 * ns * beta;
       const double cb = std::cos(beta), sb = std::sin(beta), ch = std::cos(half), sh = std::sin(half);
@@ -248,10 +298,10 @@ int mrstat_set_slice_profile(mrstat_plan* plan, const mrstat_slice_profile* prof
         t = ch * x - sh * y;  // rewinder
         y = sh * x + ch * y;
         x = t;
-        float* R = rot.data() + ((size_t)n * 32 + k) * 9 + 3 * c;
+        float* R = rot.data() + (((size_t)n * pairs + kk / 2) * kRotStride + 3 * c) * 2 + (kk & 1);
         R[0] = (float)x;
-        R[1] = (float)y;
-        R[2] = (float)z;
+        R[2] = (float)y;
+        R[4] = (float)z;
       }
     }
   e = cudaMemcpy(p->slice_rot, rot.data(), rot.size() * sizeof(float), cudaMemcpyHostToDevice);
