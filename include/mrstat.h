@@ -111,8 +111,8 @@ typedef struct mrstat_plan_info_t {
  * Create a plan: validates the sequence, builds the per-TR rotation and phase
  * tables and allocates the small work buffers (x-DFT matrices, reduction scratch,
  * CG vectors).  The large buffers are allocated by the first call that needs them:
- * the cached time courses D (3 x ntr_padded x nv float32, 4 x with B1 estimated) by
- * mrstat_linearize, the
+ * the time courses D (3 x ntr_padded x nv float32, 4 x with B1 estimated; filled by
+ * mrstat_timecourses where the linearisation keeps states instead) by mrstat_linearize, the
  * m_y scratch (ntr_padded x nv float32) by mrstat_forward / mrstat_forward_ckpt.  Synchronises the current device once.  On failure *out is
  * set to NULL.  form: a mrstat_form, optionally | MRSTAT_ESTIMATE_B1.
  * Errors: INVALID_ARG (null seq/out/arrays, bad form, non-finite or
@@ -149,8 +149,12 @@ int mrstat_plan_inject_grid_stall(mrstat_plan* plan, int32_t block);
 /*
  * Linearise the model at alpha (Algorithm 2 step 1 for every voxel, with the
  * forward-mode derivatives of Supporting Information S2): runs the Bloch recursion
- * of every voxel and caches m_y and dm_y/dln T1, dm_y/dln T2 at every echo, plus
- * rho and the mask, for later mrstat_jvp / mrstat_jhw / mrstat_timecourses calls.
+ * of every voxel and keeps what later mrstat_jvp / mrstat_jhw / mrstat_timecourses calls
+ * need: with hard pulses, no B1 map and ny <= 256 the relaxation factors and the states
+ * before up to eight segments of the train (the products re-run the recursion, as the
+ * paper does inside every product: Algorithms 2 and 4), otherwise m_y and dm_y/dln T1,
+ * dm_y/dln T2 at every echo; plus rho and the mask.  Both give the same products up to
+ * float32 rounding.
  *   alpha: device float [npar][nv] (see top; row 4 = B1 when B1 is estimated, and then
  *          a fourth channel dm_y/dB1 is cached).
  *   b1:    device float [nv] relative transmit field, or NULL for B1 = 1 (must be NULL
@@ -188,7 +192,8 @@ int mrstat_jvp(mrstat_plan* plan, const float* v, float* jv, void* stream);
 int mrstat_jhw(mrstat_plan* plan, const float* w, float* g, void* stream);
 
 /*
- * Copy one cached time course channel out of the plan: channel 0 = m_y, 1 =
+ * Copy one time course channel of the linearisation out of the plan (a linearisation that
+ * keeps states fills its time courses at the first such call): channel 0 = m_y, 1 =
  * dm_y/dln T1, 2 = dm_y/dln T2 (3 = dm_y/dB1 when B1 is estimated) at every echo (the echo signal is i * m_y because
  * the RF phases 0/180 keep m_x = 0; Supporting Information S2).
  *   out: device float [ntr][nv].  Masked-out voxels read as 0.
@@ -197,15 +202,15 @@ int mrstat_jhw(mrstat_plan* plan, const float* w, float* g, void* stream);
 int mrstat_timecourses(mrstat_plan* plan, int32_t channel, float* out, void* stream);
 
 /*
- * Recompute form of the exact model.  The paper evaluates every matrix-free product by
- * running the Bloch simulation again (Algorithms 2 and 4); with segment > 0 the plan does
- * the same instead of caching the time courses: mrstat_linearize keeps, per voxel, the
+ * Recompute form of the exact model with a chosen segment length, also for a B1 map.  The
+ * paper evaluates every matrix-free product by running the Bloch simulation again
+ * (Algorithms 2 and 4); with segment > 0 the plan does the same: mrstat_linearize keeps, per voxel, the
  * relaxation factors and the Bloch state (m_y, m_z and their ln T1 / ln T2 tangents)
  * before every segment-th TR (6 floats per voxel and segment), and every mrstat_jvp,
  * mrstat_jhw, mrstat_jhjv and mrstat_cg_fixed product re-runs the recursion from those
  * states, all segments in parallel, fused with the phase-encode sums (and, for
  * Re(J^H J) v with nkx == nx, with both of them in one pass).  The results are those of
- * the cached form up to float32 rounding.  segment = 0 restores the cached time courses.
+ * the cached form up to float32 rounding.  segment = 0 restores the default form (mrstat_linearize).
  * Either way the cached linearisation is dropped.  Synchronises the plan's device.
  *   segment: TRs per segment (>= 0; values above ntr mean one segment).
  * The recompute form needs ny <= 256, B1 known or 1 (not estimated) and hard pulses
@@ -219,7 +224,8 @@ int mrstat_set_recompute(mrstat_plan* plan, int32_t segment);
  *
  * mrstat_forward_ckpt computes s like mrstat_forward and keeps, instead of the time
  * courses, the full Bloch state of every voxel (m_y, m_z and their ln T1 / ln T2
- * tangents) before every `interval`-th TR: 6 * ceil(ntr / interval) floats per voxel.
+ * tangents) before every `interval`-th TR (fewer where longer segments balance the products
+ * better): at most 6 * ceil(ntr / interval) floats per voxel.
  * mrstat_jhw_ckpt then returns Re(J_s^H w) at that point by re-running each segment of
  * the recursion from its checkpoint (Supporting Information S2), all segments in
  * parallel, fused with the inner products of Algorithm 4; no time course is stored.

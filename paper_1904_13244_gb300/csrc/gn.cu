@@ -524,7 +524,6 @@ cudaError_t ensure_workspace(Plan* p) {
     if (e == cudaSuccess) e = r;
   };
   const size_t npv = (size_t)p->npar * nv;
-  chk(dalloc(p, &p->D2, (size_t)p->nch * p->nq * nv));
   chk(dalloc(p, &p->rho2, nv));
   chk(dalloc(p, &p->gn_g, npv));
   chk(dalloc(p, &p->gn_z, npv));
@@ -618,14 +617,15 @@ struct Solver {
     return e == cudaSuccess ? MRSTAT_OK : cuda_fail(e, "step norm");
   }
 
-  // The exact least-squares rho at the current (uniform) linearisation, nkx = nx and
-  // ny <= ntr (the k-space work arrays hold ny rows); solution rows 2..3 of gn_z
-  int ls_rho(const float* d) {
+  // The exact least-squares rho at a uniform point, nkx = nx and ny <= ntr (the k-space work
+  // arrays hold ny rows); m_n of its one time course in D (voxel stride nvd); solution rows
+  // 2..3 of gn_z
+  int ls_rho(const float* d, int nvd) {
     const int nx = p->nx, ny = p->ny, nkx = p->nkx;
     cudaError_t e = cudaMemsetAsync(p->gn_z, 0, (size_t)p->npar * p->nv * sizeof(float), st);
     if (e == cudaSuccess)
       e = vec([&] {
-        rho_ls_kspace_kernel<<<ny, 256, 0, st>>>(reinterpret_cast<const float*>(p->D), p->nv,
+        rho_ls_kspace_kernel<<<ny, 256, 0, st>>>(reinterpret_cast<const float*>(p->D), nvd,
                                                  reinterpret_cast<const float2*>(d), nkx, p->ky_ptr, p->ky_tr,
                                                  p->gn_jv);
       });
@@ -794,8 +794,22 @@ int mrstat_gn_solve(mrstat_plan* plan_, const float* d, float* alpha, const floa
                                          (float)std::log(o->t2_init_ms));
     });
     if (e != cudaSuccess) return cuda_fail(e, "rho init fill");
-    status = do_linearize(p, p->gn_alpha, b1, nullptr, p->D, p->rho, st);
-    if (status == MRSTAT_OK) status = o->rho_init_exact ? S.ls_rho(d) : S.cgls_rho(d, o->rho_init_iters);
+    if (o->rho_init_exact && rx_applies(p, b1)) {
+      // one voxel's time course serves all of them
+      e = S.vec([&] {
+        fill_rows_kernel<<<1, 32, 0, st>>>(p->gn_trial, 1, p->npar, (float)std::log(o->t1_init_ms),
+                                           (float)std::log(o->t2_init_ms));
+      });
+      if (e == cudaSuccess) {
+        Span sp(p, MRSTAT_K_BLOCH, st);
+        p->d_valid = false;
+        e = launch_bloch_n(*p, p->gn_trial, nullptr, p->D, 1, st);
+      }
+      status = e == cudaSuccess ? S.ls_rho(d, 1) : cuda_fail(e, "rho init time course");
+    } else {
+      status = do_linearize(p, p->gn_alpha, b1, nullptr, false, p->rho, st);
+      if (status == MRSTAT_OK) status = o->rho_init_exact ? S.ls_rho(d, p->nv) : S.cgls_rho(d, o->rho_init_iters);
+    }
     if (status != MRSTAT_OK) return status;
     const float* x = p->gn_z + 2 * (int64_t)nv;
     if (o->mask_threshold > 0) {
@@ -836,8 +850,8 @@ int mrstat_gn_solve(mrstat_plan* plan_, const float* d, float* alpha, const floa
     return lowrank_jvp(p, p->gn_q, s_out, st);
   };
   auto exact_point = [&]() -> int {
-    int r = do_linearize(p, p->gn_alpha, b1, p->gn_mask, p->D, p->rho, st);
-    if (r == MRSTAT_OK) r = do_signal(p, p->D, p->rho, p->gn_s, st);
+    int r = do_linearize(p, p->gn_alpha, b1, p->gn_mask, false, p->rho, st);
+    if (r == MRSTAT_OK) r = do_signal(p, false, p->rho, p->gn_s, st);
     if (r == MRSTAT_OK) r = S.residual(p->gn_s, d, p->gn_r, p->gn_sc + S_F);
     return r;
   };
@@ -929,8 +943,8 @@ int mrstat_gn_solve(mrstat_plan* plan_, const float* d, float* alpha, const floa
         status = sur_signal(p->gn_trial, p->gn_st);
       }
     } else {
-      status = do_linearize(p, p->gn_trial, b1, p->gn_mask, p->D2, p->rho2, st);
-      if (status == MRSTAT_OK) status = do_signal(p, p->D2, p->rho2, p->gn_st, st);
+      status = do_linearize(p, p->gn_trial, b1, p->gn_mask, true, p->rho2, st);
+      if (status == MRSTAT_OK) status = do_signal(p, true, p->rho2, p->gn_st, st);
     }
     if (status == MRSTAT_OK) status = S.residual(p->gn_st, d, p->gn_rt, p->gn_sc + S_F);
     if (status == MRSTAT_OK) status = fetch();
@@ -952,8 +966,8 @@ int mrstat_gn_solve(mrstat_plan* plan_, const float* d, float* alpha, const floa
     local.iterations = k + 1;
     if (sur && !acc) swap_ptr(p->lr->coef, p->lr->coef2);
     if (acc) {
-      if (!sur) swap_ptr(p->D, p->D2);
-      swap_ptr(p->rho, p->rho2);
+      if (sur) swap_ptr(p->rho, p->rho2);
+      else swap_linearisations(p);
       swap_ptr(p->gn_alpha, p->gn_trial);
       swap_ptr(p->gn_s, p->gn_st);
       swap_ptr(p->gn_r, p->gn_rt);

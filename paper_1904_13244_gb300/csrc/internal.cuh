@@ -24,6 +24,14 @@ constexpr int kRedBlocks = 608;
 // buffers of up to eight partials per block of the persistent column kernels
 constexpr int kRedSlots = 16 * kRedBlocks;
 
+// A linearisation by recomputation (recur.cu): relaxation factors and the Bloch states before
+// every seg-th TR, column-major.
+struct RxLin {
+  float* fac = nullptr;  // [6][nx][nys]
+  float* st = nullptr;   // [nseg][ns][nx][nys]
+  int seg = 0, nseg = 0, ns = 6;
+};
+
 struct Plan {
   int nx = 0, ny = 0, nkx = 0, ntr = 0;
   int ntr_pad = 0;   // ntr rounded up to a multiple of 4
@@ -39,6 +47,7 @@ struct Plan {
   // per-TR tables (device)
   float2* cs = nullptr;     // [ntr_pad] (cos phi_n, sin phi_n), phi_n the signed flip
   float* phi = nullptr;     // [ntr_pad] signed flip (radians)
+  float4* csp = nullptr;    // [ntr_pad][2] (c, c, s, s), (-s, -s, 0, 0) of the signed flip
   // slice profile (mrstat_set_slice_profile): 0 isochromats = hard pulses
   int slice_iso = 0, slice_sub = 0;
   float* slice_rot = nullptr;    // [ntr_pad][pairs][10][2] composed pulses of each TR and isochromat pair (slice.cu)
@@ -95,7 +104,19 @@ struct Plan {
   LowRank* lr = nullptr;            // low-rank form (after mrstat_lowrank_set_basis)
   int* dev_err = nullptr;           // set by a kernel whose bounded wait ran out
 
-  // checkpointed form
+  // recomputed linearisations of the exact model (hard pulses, no B1 map): the plan's, the
+  // Gauss-Newton trial point's, the forward's (m alone) and the checkpointed forward's
+  RxLin rx, rx2, rxf, rxc;
+  int rx_seg = 0;                   // TRs per segment
+  bool rx_active = false;           // the current exact linearisation is rx (else D)
+  bool d_valid = false;             // D holds its time courses
+  unsigned* rx_ticket = nullptr;    // zero between launches
+  float4* rx_etab = nullptr;        // [ny][row pairs] phases (recur.cu)
+  float2* rxc_rho = nullptr;        // [nv] masked rho and mask of the checkpointed forward
+  float* rxc_maskf = nullptr;
+  bool rxc_active = false;          // the checkpointed forward kept rxc (else ckpt)
+
+  // checkpointed form with a B1 map
   float* ckpt = nullptr;        // [nseg][6][nv] Bloch states at segment starts
   float* zpart = nullptr;       // [nseg][6][nv] per-segment partial inner products
   int ckpt_interval = 0, ckpt_nseg = 0, ckpt_cap = 0;
@@ -200,9 +221,15 @@ struct Span {
 // product building blocks on a plan (plan.cu); they return an mrstat_status
 int do_jvp(Plan* p, const float* v, float2* jv, cudaStream_t st);
 int do_jhw(Plan* p, const float2* w, float* g, cudaStream_t st);
-int do_signal(Plan* p, const float4* D, const float2* rho_masked, float2* s, cudaStream_t st);
-int do_linearize(Plan* p, const float* alpha, const float* b1, const uint8_t* mask, float4* D,
-                 float2* rho, cudaStream_t st);
+// the exact linearisation at alpha: the plan's, or (trial) the Gauss-Newton trial point's
+int do_linearize(Plan* p, const float* alpha, const float* b1, const uint8_t* mask, bool trial, float2* rho,
+                 cudaStream_t st);
+// the signal of one of them, with its masked rho
+int do_signal(Plan* p, bool trial, const float2* rho_masked, float2* s, cudaStream_t st);
+// whether the exact model runs by recomputation (recur.cu) at this B1 map
+bool rx_applies(const Plan* p, const float* b1);
+// exchange the two (an accepted step)
+void swap_linearisations(Plan* p);
 cudaError_t do_dot(Plan* p, const float* a, const float* b, int64_t n, double* out, cudaStream_t st);
 // Re(J^H J) v with the plan's active linearisation (exact: J.v then J^H; low-rank: per-ky
 // Gram); with vdot also *vdot = <v, Re(J^H J) v> and with vv also *vv = <v, v> (fused into
@@ -286,6 +313,20 @@ cudaError_t launch_ycontract(const Plan& p, const float4* D, int nch, cudaStream
 // g from W~ = p.wt, or from wt (then times scale) when given
 cudaError_t launch_jhw_dot(const Plan& p, float* g, cudaStream_t st, const float2* wt = nullptr, float scale = 1.f);
 cudaError_t launch_timecourse(const Plan& p, int channel, float* out, cudaStream_t st);
+// recur.cu: the exact model by recomputation
+inline int rx_nys(const Plan& p) { return (p.ny + 1) / 2 * 2; }
+bool rx_supported(const Plan& p);
+int rx_segment(const Plan& p, int sms);
+std::vector<float4> rx_phase_table(const Plan& p, const std::vector<float2>& roots);
+cudaError_t launch_rx_states(const Plan& p, const RxLin& L, const float* alpha, const uint8_t* mask, float2* rho,
+                             float* maskf, cudaStream_t st);
+cudaError_t launch_rx_signal(const Plan& p, const RxLin& L, const float2* rho, cudaStream_t st);
+cudaError_t launch_rx_jv(const Plan& p, const RxLin& L, const float* v, cudaStream_t st);
+cudaError_t launch_rx_jhw(const Plan& p, const RxLin& L, const float2* rho, const float* maskf, const float2* wt,
+                          float* g, cudaStream_t st);
+cudaError_t launch_rx_jhjv(const Plan& p, const RxLin& L, const float* v, float* g, double* vdot, double* vv,
+                           cudaStream_t st);
+cudaError_t launch_rx_expand(const Plan& p, const RxLin& L, float4* D, cudaStream_t st);
 // dft.cu
 cudaError_t launch_cgemm(const float2* A, const float2* B, float2* C, int M, int N, int K,
                          const int* gate, cudaStream_t st);

@@ -46,7 +46,8 @@ void free_plan(Plan* p) {
                   p->gn_dir, p->gn_q, p->gn_alpha, p->gn_trial, p->gn_s, p->gn_r, p->gn_st,
                   p->gn_rt, p->gn_jv, p->gn_mask, p->gn_sc, p->gn_si, p->bf_ft_hi, p->bf_ft_lo,
                   p->bf_fh_hi, p->bf_fh_lo, p->bf_a_hi, p->bf_a_lo, p->bf_w_hi, p->bf_w_lo, p->dev_err, p->ckpt, p->zpart,
-                  p->rc_rlx, p->rc_ckpt, p->rc_gpart, p->rc_b1};
+                  p->rc_rlx, p->rc_ckpt, p->rc_gpart, p->rc_b1, p->csp, p->rx.fac, p->rx.st, p->rx2.fac, p->rx2.st,
+                  p->rxf.fac, p->rxf.st, p->rxc.fac, p->rxc.st, p->rx_ticket, p->rx_etab, p->rxc_rho, p->rxc_maskf};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   for (cudaEvent_t e : p->event_pool) cudaEventDestroy(e);
@@ -80,6 +81,35 @@ cudaError_t ensure_forward_scratch(Plan* p) {
   if (p->dfwd != nullptr) return cudaSuccess;
   return dalloc(p, &p->dfwd, (size_t)p->nq * p->nv);
 }
+
+// the exact model at hard pulses without a B1 map runs by recomputation
+bool rx_applies(const Plan* p, const float* b1) {
+  return p->rx_seg > 0 && p->slice_iso == 0 && p->rc_seg == 0 && b1 == nullptr;
+}
+
+namespace {
+
+// Allocates L (once per segment length) with ns floats per state.
+cudaError_t ensure_rx(Plan* p, RxLin* L, int ns, int seg) {
+  const size_t nvp = (size_t)p->nx * rx_nys(*p);
+  const int nseg = (p->ntr + seg - 1) / seg;
+  cudaError_t e = cudaSuccess;
+  if (L->fac == nullptr) e = dalloc(p, &L->fac, 6 * nvp);
+  if (e == cudaSuccess && L->st != nullptr && L->nseg < nseg) {
+    e = cudaDeviceSynchronize();
+    cudaFree(L->st);
+    p->bytes -= (int64_t)((size_t)L->nseg * L->ns * nvp * sizeof(float));
+    L->st = nullptr;
+  }
+  if (e == cudaSuccess && L->st == nullptr) {
+    e = dalloc(p, &L->st, (size_t)nseg * ns * nvp);
+    L->ns = ns;
+    L->nseg = nseg;
+  }
+  return e;
+}
+
+}  // namespace
 
 int build_split_tables(Plan* p) {
   if (p->tc != nullptr) return MRSTAT_OK;
@@ -165,6 +195,14 @@ int do_jvp(Plan* p, const float* v, float2* jv, cudaStream_t st) {
     if (e != cudaSuccess) return cuda_fail(e, "recompute J.v launch");
     return do_xdft(p, p->A, jv, p->gate, st);
   }
+  if (p->rx_active) {
+    {
+      Span sp(p, MRSTAT_K_YCONTRACT, st);
+      e = launch_rx_jv(*p, p->rx, v, st);
+    }
+    if (e != cudaSuccess) return cuda_fail(e, "J.v launch");
+    return do_xdft(p, p->A, jv, p->gate, st);
+  }
   {
     Span sp(p, MRSTAT_K_VECTOR, st);
     e = launch_prep_jvp(*p, v, st);
@@ -191,14 +229,22 @@ int do_jhw(Plan* p, const float2* w, float* g, cudaStream_t st) {
   }
   {
     Span sp(p, MRSTAT_K_JHW_DOT, st);
-    e = launch_jhw_dot(*p, g, st);
+    e = p->rx_active ? launch_rx_jhw(*p, p->rx, p->rho, p->maskf, p->wt, g, st) : launch_jhw_dot(*p, g, st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "jhw_dot launch");
   return MRSTAT_OK;
 }
 
-int do_signal(Plan* p, const float4* D, const float2* rho_masked, float2* s, cudaStream_t st) {
+int do_signal(Plan* p, bool trial, const float2* rho_masked, float2* s, cudaStream_t st) {
   cudaError_t e;
+  if (p->rx_active) {
+    {
+      Span sp(p, MRSTAT_K_YCONTRACT, st);
+      e = launch_rx_signal(*p, trial ? p->rx2 : p->rx, rho_masked, st);
+    }
+    if (e != cudaSuccess) return cuda_fail(e, "signal launch");
+    return do_xdft(p, p->A, s, nullptr, st);
+  }
   {
     Span sp(p, MRSTAT_K_VECTOR, st);
     e = launch_prep_rho(*p, rho_masked, st);
@@ -207,10 +253,17 @@ int do_signal(Plan* p, const float4* D, const float2* rho_masked, float2* s, cud
   {
     // the signal only needs channel 0 (m_y) and coefficient 0 (rho)
     Span sp(p, MRSTAT_K_YCONTRACT, st);
-    e = launch_ycontract(*p, D, 1, st);
+    e = launch_ycontract(*p, trial ? p->D2 : p->D, 1, st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "ycontract launch");
   return do_xdft(p, p->A, s, nullptr, st);
+}
+
+void swap_linearisations(Plan* p) {
+  if (p->rx_active) std::swap(p->rx, p->rx2);  // D stays: it is only filled on demand
+  else std::swap(p->D, p->D2);
+  std::swap(p->rho, p->rho2);
+  p->d_valid = false;
 }
 
 int do_xdft(Plan* p, const float2* A, float2* out, const int* gate, cudaStream_t st) {
@@ -251,9 +304,24 @@ int do_xdft_adj(Plan* p, const float2* w, float2* out, const int* gate, cudaStre
   return e == cudaSuccess ? MRSTAT_OK : cuda_fail(e, "x-DFT adjoint launch");
 }
 
-int do_linearize(Plan* p, const float* alpha, const float* b1, const uint8_t* mask, float4* D,
-                 float2* rho, cudaStream_t st) {
+int do_linearize(Plan* p, const float* alpha, const float* b1, const uint8_t* mask, bool trial, float2* rho,
+                 cudaStream_t st) {
   cudaError_t e;
+  p->rx_active = rx_applies(p, b1);
+  if (!trial) p->d_valid = false;
+  if (p->rx_active) {
+    RxLin* L = trial ? &p->rx2 : &p->rx;
+    e = ensure_rx(p, L, 6, p->rx_seg);
+    if (e != cudaSuccess) return cuda_fail(e, "linearisation allocation");
+    Span sp(p, MRSTAT_K_BLOCH, st);
+    L->seg = p->rx_seg;
+    e = launch_rx_states(*p, *L, alpha, mask, rho, p->maskf, st);
+    return e == cudaSuccess ? MRSTAT_OK : cuda_fail(e, "linearisation launch");
+  }
+  if (trial && p->D2 == nullptr) {
+    e = dalloc(p, &p->D2, (size_t)p->nch * p->nq * p->nv);
+    if (e != cudaSuccess) return cuda_fail(e, "time-course allocation");
+  }
   {
     Span sp(p, MRSTAT_K_VECTOR, st);
     e = launch_prep_linearize(*p, alpha, mask, rho, st);
@@ -261,12 +329,14 @@ int do_linearize(Plan* p, const float* alpha, const float* b1, const uint8_t* ma
   if (e != cudaSuccess) return cuda_fail(e, "prep_linearize launch");
   if (p->slice_iso > 0 && b1 != nullptr)
     return fail(MRSTAT_ERR_UNSUPPORTED, "the slice-profile model takes B1 = 1 (no map)");
+  float4* D = trial ? p->D2 : p->D;
   {
     Span sp(p, MRSTAT_K_BLOCH, st);
     e = p->slice_iso > 0 ? launch_bloch_slice(*p, alpha, mask, D, 3, st)
                          : launch_bloch(*p, alpha, b1, mask, D, p->nch, st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "bloch launch");
+  if (!trial) p->d_valid = true;
   return MRSTAT_OK;
 }
 
@@ -275,6 +345,13 @@ int do_linearize(Plan* p, const float* alpha, const float* b1, const uint8_t* ma
 // W~ = nx A and the two x-DFTs are skipped: exact, not an approximation.
 int do_jhjv(Plan* p, const float* v, float* out, cudaStream_t st, double* vdot, double* vv) {
   if (p->lr && p->lr->active) return lowrank_jhjv(p, v, out, st, vdot, vv);
+  if (p->nkx == p->nx && p->rc_seg == 0 && p->rx_active && (vdot != nullptr || vv == nullptr)) {
+    // the simulation, both phase-encode sums, the tangent products and the inner products
+    // in one pass
+    Span sp(p, MRSTAT_K_JHW_DOT, st);
+    const cudaError_t e = launch_rx_jhjv(*p, p->rx, v, out, vdot, vv, st);
+    return e == cudaSuccess ? MRSTAT_OK : cuda_fail(e, "J^H J v launch");
+  }
   if (vv != nullptr) {
     const int s = do_jhjv(p, v, out, st, vdot);
     if (s != MRSTAT_OK) return s;
@@ -458,6 +535,7 @@ int mrstat_plan_create(const mrstat_seq* seq, int32_t form, mrstat_plan** out) {
 
   // host tables (float64, rounded once)
   std::vector<float2> cs(p->ntr_pad);
+  std::vector<float4> csp(2 * (size_t)p->ntr_pad);
   std::vector<float> phi(p->ntr_pad, 0.f);
   std::vector<int> kyi(p->ntr_pad, 0);
   for (int n = 0; n < p->ntr_pad; ++n) {
@@ -469,6 +547,8 @@ int mrstat_plan_create(const mrstat_seq* seq, int32_t form, mrstat_plan** out) {
     }
     phi[n] = (float)ph;
     cs[n] = make_float2((float)std::cos(ph), (float)std::sin(ph));
+    csp[2 * n] = make_float4(cs[n].x, cs[n].x, cs[n].y, cs[n].y);
+    csp[2 * n + 1] = make_float4(-cs[n].y, -cs[n].y, 0.f, 0.f);
   }
   std::vector<int> ky_ptr(p->ny + 1, 0), ky_tr(std::max(p->ntr, 1), 0);
   for (int n = 0; n < p->ntr; ++n) ky_ptr[kyi[n] + 1]++;
@@ -486,12 +566,22 @@ int mrstat_plan_create(const mrstat_seq* seq, int32_t form, mrstat_plan** out) {
       unit_root(kx * ix, p->nx, &fh[(size_t)k * p->nx + ix], true);
     }
 
+  std::vector<float4> rx_etab;
   const size_t nv = p->nv, nq = p->nq;
   cudaError_t e = cudaSuccess;
   auto chk = [&](cudaError_t r) {
     if (e == cudaSuccess) e = r;
   };
   chk(dalloc(p, &p->cs, p->ntr_pad));
+  chk(dalloc(p, &p->csp, csp.size()));
+  if (rx_supported(*p)) {
+    int sms = 0;
+    chk(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device));
+    p->rx_seg = rx_segment(*p, sms);
+    chk(dalloc(p, &p->rx_ticket, 1));
+    rx_etab = rx_phase_table(*p, roots);
+    chk(dalloc(p, &p->rx_etab, rx_etab.size()));
+  }
   chk(dalloc(p, &p->phi, p->ntr_pad));
   chk(dalloc(p, &p->kyi, p->ntr_pad));
   chk(dalloc(p, &p->roots, p->ny));
@@ -521,6 +611,10 @@ int mrstat_plan_create(const mrstat_seq* seq, int32_t form, mrstat_plan** out) {
     return st;
   }
   chk(cudaMemcpy(p->cs, cs.data(), cs.size() * sizeof(float2), cudaMemcpyHostToDevice));
+  chk(cudaMemcpy(p->csp, csp.data(), csp.size() * sizeof(float4), cudaMemcpyHostToDevice));
+  if (p->rx_etab)
+    chk(cudaMemcpy(p->rx_etab, rx_etab.data(), rx_etab.size() * sizeof(float4), cudaMemcpyHostToDevice));
+  if (p->rx_ticket) chk(cudaMemset(p->rx_ticket, 0, sizeof(unsigned)));
   chk(cudaMemcpy(p->phi, phi.data(), phi.size() * sizeof(float), cudaMemcpyHostToDevice));
   chk(cudaMemcpy(p->kyi, kyi.data(), kyi.size() * sizeof(int), cudaMemcpyHostToDevice));
   chk(cudaMemcpy(p->roots, roots.data(), roots.size() * sizeof(float2), cudaMemcpyHostToDevice));
@@ -603,7 +697,7 @@ int mrstat_linearize(mrstat_plan* plan, const float* alpha, const float* b1, con
   }
   cudaError_t ea = ensure_timecourses(plan);
   if (ea != cudaSuccess) return cuda_fail(ea, "time-course allocation");
-  const int status = do_linearize(plan, alpha, b1, mask, plan->D, plan->rho, st);
+  const int status = do_linearize(plan, alpha, b1, mask, false, plan->rho, st);
   if (status != MRSTAT_OK) return status;
   plan->linearized = true;
   return MRSTAT_OK;
@@ -620,7 +714,25 @@ int mrstat_forward(mrstat_plan* plan, const float* alpha, const float* b1, const
     return fail(MRSTAT_ERR_UNSUPPORTED, "the slice-profile model takes B1 = 1 (no map)");
   DeviceGuard g(plan->device);
   cudaStream_t st = as_stream(stream);
-  cudaError_t e = ensure_forward_scratch(plan);
+  cudaError_t e;
+  if (plan->npar == 4 && plan->rx_seg > 0 && plan->slice_iso == 0 && b1 == nullptr) {
+    // states of m alone, then every segment's share of the phase-encode sums
+    e = ensure_rx(plan, &plan->rxf, 2, plan->rx_seg);
+    if (e != cudaSuccess) return cuda_fail(e, "forward scratch allocation");
+    plan->rxf.seg = plan->rx_seg;
+    {
+      Span sp(plan, MRSTAT_K_BLOCH, st);
+      e = launch_rx_states(*plan, plan->rxf, alpha, mask, plan->cf, nullptr, st);
+    }
+    if (e != cudaSuccess) return cuda_fail(e, "bloch launch");
+    {
+      Span sp(plan, MRSTAT_K_YCONTRACT, st);
+      e = launch_rx_signal(*plan, plan->rxf, plan->cf, st);
+    }
+    if (e != cudaSuccess) return cuda_fail(e, "signal launch");
+    return do_xdft(plan, plan->A, reinterpret_cast<float2*>(s), nullptr, st);
+  }
+  e = ensure_forward_scratch(plan);
   if (e != cudaSuccess) return cuda_fail(e, "forward scratch allocation");
   {
     Span sp(plan, MRSTAT_K_BLOCH, st);
@@ -670,6 +782,12 @@ int mrstat_timecourses(mrstat_plan* plan, int32_t channel, float* out, void* str
   if (!plan->linearized || plan->D == nullptr || (plan->lr && plan->lr->active))
     return fail(MRSTAT_ERR_NOT_LINEARIZED, "timecourses need an exact mrstat_linearize");
   DeviceGuard g(plan->device);
+  if (plan->rx_active && !plan->d_valid) {  // all channels, from the kept states
+    Span sp(plan, MRSTAT_K_BLOCH, as_stream(stream));
+    const cudaError_t e = launch_rx_expand(*plan, plan->rx, plan->D, as_stream(stream));
+    if (e != cudaSuccess) return cuda_fail(e, "timecourse launch");
+    plan->d_valid = true;
+  }
   Span sp(plan, MRSTAT_K_VECTOR, as_stream(stream));
   cudaError_t e = launch_timecourse(*plan, channel, out, as_stream(stream));
   return e == cudaSuccess ? MRSTAT_OK : cuda_fail(e, "timecourse launch");
@@ -696,7 +814,33 @@ int mrstat_forward_ckpt(mrstat_plan* plan, const float* alpha, const float* b1, 
   if (plan->slice_iso > 0) return fail(MRSTAT_ERR_UNSUPPORTED, "the checkpointed form uses the hard-pulse model");
   DeviceGuard g(plan->device);
   cudaStream_t st = as_stream(stream);
-  cudaError_t e = ensure_forward_scratch(plan);
+  cudaError_t e;
+  plan->ckpt_ready = false;
+  plan->rxc_active = plan->rx_seg > 0 && b1 == nullptr;
+  if (plan->rxc_active) {
+    // states every seg-th TR, with the tangents: at most one per interval TRs
+    const int seg = std::max(std::min(interval, plan->ntr_pad), plan->rx_seg);
+    e = ensure_rx(plan, &plan->rxc, 6, seg);
+    if (e == cudaSuccess && plan->rxc_rho == nullptr) e = dalloc(plan, &plan->rxc_rho, (size_t)plan->nv);
+    if (e == cudaSuccess && plan->rxc_maskf == nullptr) e = dalloc(plan, &plan->rxc_maskf, (size_t)plan->nv);
+    if (e != cudaSuccess) return cuda_fail(e, "checkpoint allocation");
+    plan->rxc.seg = seg;
+    plan->rxc.nseg = (plan->ntr + seg - 1) / seg;
+    {
+      Span sp(plan, MRSTAT_K_BLOCH, st);
+      e = launch_rx_states(*plan, plan->rxc, alpha, mask, plan->rxc_rho, plan->rxc_maskf, st);
+    }
+    if (e != cudaSuccess) return cuda_fail(e, "checkpointed Bloch launch");
+    {
+      Span sp(plan, MRSTAT_K_YCONTRACT, st);
+      e = launch_rx_signal(*plan, plan->rxc, plan->rxc_rho, st);
+    }
+    if (e != cudaSuccess) return cuda_fail(e, "signal launch");
+    const int status = do_xdft(plan, plan->A, reinterpret_cast<float2*>(s), nullptr, st);
+    plan->ckpt_ready = status == MRSTAT_OK;
+    return status;
+  }
+  e = ensure_forward_scratch(plan);
   if (e != cudaSuccess) return cuda_fail(e, "forward scratch allocation");
   const int nseg = (plan->ntr + interval - 1) / interval;
   if (nseg > plan->ckpt_cap) {
@@ -751,6 +895,11 @@ int mrstat_jhw_ckpt(mrstat_plan* plan, const float* w, float* gout, void* stream
   int status = do_xdft_adj(plan, reinterpret_cast<const float2*>(w), plan->wt, nullptr, st);
   if (status != MRSTAT_OK) return status;
   cudaError_t e;
+  if (plan->rxc_active) {
+    Span sp(plan, MRSTAT_K_JHW_DOT, st);
+    e = launch_rx_jhw(*plan, plan->rxc, plan->rxc_rho, plan->rxc_maskf, plan->wt, gout, st);
+    return e == cudaSuccess ? MRSTAT_OK : cuda_fail(e, "segment recompute launch");
+  }
   {
     Span sp(plan, MRSTAT_K_JHW_DOT, st, 1, 2);  // the segment kernel and the segment sum
     e = launch_segment_jhw(*plan, plan->ckpt_alpha, plan->ckpt_b1, plan->ckpt_mask, plan->ckpt_interval,
