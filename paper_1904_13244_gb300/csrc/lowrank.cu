@@ -29,6 +29,7 @@
 
 #include "internal.cuh"
 #include "lowrank.cuh"
+#include "packed.cuh"
 #include "reduce.cuh"
 #include "steihaug.cuh"
 
@@ -42,18 +43,36 @@ __device__ __forceinline__ void put_split(__nv_bfloat16* hi, __nv_bfloat16* lo, 
 }
 
 // ---------------------------------------------------------------------------
-// exact linearisation projected onto U: Bloch recursion with tangents (as bloch.cu),
-// accumulating c_r += U[n][r] m_y, dc1_r += U[n][r] dm_y/dlnT1, dc2_r += U[n][r] dm_y/dlnT2
+// exact linearisation projected onto U: Bloch recursion with tangents (Supporting
+// Information S2), accumulating the sums over the TRs of U[n][r] times the rotated m_y and its
+// ln T1 and ln T2 tangents.  The echo lies TE after the pulse: m_y = E y, and the tangents
+// E a and E b + D y with E = E2(TE), D = dE/dln T2, constants of the voxel that the finished
+// sums take; the relaxations over TE and TR - TE act as one step over TR.
+//
+// Bound by the FP32 pipe: 3 R multiply-adds of the projection (in packed pairs of basis
+// functions) and 21 of the recursion per voxel and TR, one voxel per thread.  The rows of U
+// and the pulse table come through shared memory two chunks deep (read from global memory
+// per TR, the pulse table alone cost an L2 latency every few TRs).  Blocks of two warps: a
+// block outside the mask ends at once, so the warps that count spread over the SMs.  At 224 x
+// 224, 1120 TRs and R = 32: 288 us, 489 before (scalar sums, two decays, tables from global
+// memory).  Tried: the basis functions of a voxel split over two warps (352 us), rows of U
+// prefetched into registers (302), seven blocks per SM at 146 registers (297).
 // ---------------------------------------------------------------------------
-template <int R>
-__global__ void __launch_bounds__(128)
+constexpr int kProjThreads = 64, kProjChunk = 32;
+constexpr int kProjBlocks = 5;  // per SM: up to 204 registers, of which R = 32 holds 96 in sums
+
+template <int R, bool B1MAP>
+__global__ void __launch_bounds__(kProjThreads, kProjBlocks)
 lr_project_kernel(const float* __restrict__ alpha, const float* __restrict__ b1,
                   const uint8_t* __restrict__ mask, const float2* __restrict__ cs, const float* __restrict__ phi,
-                  const float* __restrict__ U, int nv, int ntr, float te, float tb, float m0z,
+                  const float* __restrict__ U, int nv, int ntr, float te, float tr, float m0z,
                   float* __restrict__ coef) {
-  constexpr int CH = 64;  // TRs of U staged per chunk
-  __shared__ __align__(16) float us[CH * R];
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  using pk::f2;
+  constexpr int CH = kProjChunk;
+  __shared__ __align__(16) float us[2][CH * R];  // rows of U
+  __shared__ __align__(16) float2 ps[2][CH];     // (cos, sin) of the pulse, or with a B1 map its angle
+  const int tid = threadIdx.x;
+  const int j = blockIdx.x * kProjThreads + tid;
   const bool valid = j < nv;
   const bool on = valid && (mask == nullptr || mask[j] != 0);
   // a block whose voxels all lie outside the mask has only zeros to write
@@ -66,31 +85,36 @@ lr_project_kernel(const float* __restrict__ alpha, const float* __restrict__ b1,
   if (valid) {
     t1 = expf(alpha[j]);
     t2 = expf(alpha[nv + j]);
-    if (b1 != nullptr) bj = b1[j];
+    if (B1MAP) bj = b1[j];
   }
-  const float ra1 = te / t1, ra2 = te / t2, rb1 = tb / t1, rb2 = tb / t2;
-  const float x1a = expm1f(-ra1), x2a = expm1f(-ra2), x1b = expm1f(-rb1), x2b = expm1f(-rb2);
-  const float d1a = ra1 * (1.f + x1a), d2a = ra2 * (1.f + x2a), d1b = rb1 * (1.f + x1b), d2b = rb2 * (1.f + x2b);
+  const float x1 = expm1f(-tr / t1), x2 = expm1f(-tr / t2), x2e = expm1f(-te / t2);
+  const float d1 = tr / t1 * (1.f + x1), d2 = tr / t2 * (1.f + x2);
   float my = 0.f, mz = m0z, ay = 0.f, az = 0.f, by = 0.f, bz = 0.f;
-  float c0[R], c1[R], c2[R];
+  f2 c0[R / 2], c1[R / 2], c2[R / 2];
 #pragma unroll
-  for (int r = 0; r < R; ++r) c0[r] = c1[r] = c2[r] = 0.f;
+  for (int r = 0; r < R / 2; ++r) c0[r] = c1[r] = c2[r] = 0ull;
 
-  for (int n0 = 0; n0 < ntr; n0 += CH) {
+  // chunk n0 into buffer buf: R is a multiple of 8, U and the rows of a chunk 16-byte aligned
+  auto stage = [&](int n0, int buf) {
     const int cnt = min(CH, ntr - n0);
-    __syncthreads();
-    for (int e = threadIdx.x; e < cnt * R; e += blockDim.x) us[e] = U[(size_t)n0 * R + e];
-    __syncthreads();
+    for (int e = tid; e < cnt * R / 4; e += kProjThreads)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(us[buf] + 4 * e)),
+                   "l"(U + (size_t)n0 * R + 4 * e)
+                   : "memory");
+    if (tid < cnt) ps[buf][tid] = B1MAP ? make_float2(__ldg(phi + n0 + tid), 0.f) : __ldg(cs + n0 + tid);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  stage(0, 0);
+  for (int n0 = 0, buf = 0; n0 < ntr; n0 += CH, buf ^= 1) {
+    const int cnt = min(CH, ntr - n0);
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();  // this chunk is in shared memory, the previous one no longer read
+    if (n0 + CH < ntr) stage(n0 + CH, buf ^ 1);
+#pragma unroll 2
     for (int t = 0; t < cnt; ++t) {
-      const int n = n0 + t;
-      float c, s;
-      if (b1 != nullptr) {
-        sincosf(__ldg(phi + n) * bj, &s, &c);
-      } else {
-        const float2 v = __ldg(cs + n);
-        c = v.x;
-        s = v.y;
-      }
+      const float2 p = ps[buf][t];
+      float c = p.x, s = p.y;
+      if (B1MAP) sincosf(p.x * bj, &s, &c);
       float ty = c * my + s * mz;
       mz = c * mz - s * my;
       my = ty;
@@ -100,46 +124,40 @@ lr_project_kernel(const float* __restrict__ alpha, const float* __restrict__ b1,
       ty = c * by + s * bz;
       bz = c * bz - s * by;
       by = ty;
-      float zm1 = mz - 1.f;
-      ay = fmaf(x2a, ay, ay);
-      az = fmaf(x1a, az, fmaf(d1a, zm1, az));
-      by = fmaf(x2a, by, fmaf(d2a, my, by));
-      bz = fmaf(x1a, bz, bz);
-      my = fmaf(x2a, my, my);
-      mz = fmaf(x1a, zm1, mz);
-      const float4* u4 = reinterpret_cast<const float4*>(us + t * R);
+      const f2 m2 = pk::both(my), a2 = pk::both(ay), b2 = pk::both(by);
+      const ulonglong2* u2 = reinterpret_cast<const ulonglong2*>(us[buf] + t * R);
 #pragma unroll
-      for (int r4 = 0; r4 < R / 4; ++r4) {
-        const float4 u = u4[r4];
-        c0[4 * r4 + 0] = fmaf(u.x, my, c0[4 * r4 + 0]);
-        c0[4 * r4 + 1] = fmaf(u.y, my, c0[4 * r4 + 1]);
-        c0[4 * r4 + 2] = fmaf(u.z, my, c0[4 * r4 + 2]);
-        c0[4 * r4 + 3] = fmaf(u.w, my, c0[4 * r4 + 3]);
-        c1[4 * r4 + 0] = fmaf(u.x, ay, c1[4 * r4 + 0]);
-        c1[4 * r4 + 1] = fmaf(u.y, ay, c1[4 * r4 + 1]);
-        c1[4 * r4 + 2] = fmaf(u.z, ay, c1[4 * r4 + 2]);
-        c1[4 * r4 + 3] = fmaf(u.w, ay, c1[4 * r4 + 3]);
-        c2[4 * r4 + 0] = fmaf(u.x, by, c2[4 * r4 + 0]);
-        c2[4 * r4 + 1] = fmaf(u.y, by, c2[4 * r4 + 1]);
-        c2[4 * r4 + 2] = fmaf(u.z, by, c2[4 * r4 + 2]);
-        c2[4 * r4 + 3] = fmaf(u.w, by, c2[4 * r4 + 3]);
+      for (int r = 0; r < R / 4; ++r) {
+        const ulonglong2 u = u2[r];
+        c0[2 * r] = pk::fma(u.x, m2, c0[2 * r]);
+        c0[2 * r + 1] = pk::fma(u.y, m2, c0[2 * r + 1]);
+        c1[2 * r] = pk::fma(u.x, a2, c1[2 * r]);
+        c1[2 * r + 1] = pk::fma(u.y, a2, c1[2 * r + 1]);
+        c2[2 * r] = pk::fma(u.x, b2, c2[2 * r]);
+        c2[2 * r + 1] = pk::fma(u.y, b2, c2[2 * r + 1]);
       }
-      zm1 = mz - 1.f;
-      ay = fmaf(x2b, ay, ay);
-      az = fmaf(x1b, az, fmaf(d1b, zm1, az));
-      by = fmaf(x2b, by, fmaf(d2b, my, by));
-      bz = fmaf(x1b, bz, bz);
-      my = fmaf(x2b, my, my);
-      mz = fmaf(x1b, zm1, mz);
+      const float zm1 = mz - 1.f;
+      ay = fmaf(x2, ay, ay);
+      az = fmaf(x1, az, fmaf(d1, zm1, az));
+      by = fmaf(x2, by, fmaf(d2, my, by));
+      bz = fmaf(x1, bz, bz);
+      my = fmaf(x2, my, my);
+      mz = fmaf(x1, zm1, mz);
     }
   }
   if (!valid) return;
-  const float m = on ? 1.f : 0.f;
+  const float m = on ? 1.f : 0.f, ee = m * (1.f + x2e), de = m * (te / t2 * (1.f + x2e));
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    coef[(size_t)r * nv + j] = c0[r] * m;
-    coef[(size_t)(R + r) * nv + j] = c1[r] * m;
-    coef[(size_t)(2 * R + r) * nv + j] = c2[r] * m;
+  for (int r = 0; r < R / 2; ++r) {
+    const float2 y = pk::split(c0[r]), a = pk::split(c1[r]), b = pk::split(c2[r]);
+    float* o = coef + (size_t)2 * r * nv + j;
+    const size_t plane = (size_t)R * nv;
+    o[0] = ee * y.x;
+    o[nv] = ee * y.y;
+    o[plane] = ee * a.x;
+    o[plane + nv] = ee * a.y;
+    o[2 * plane] = fmaf(ee, b.x, de * y.x);
+    o[2 * plane + nv] = fmaf(ee, b.y, de * y.y);
   }
 }
 
@@ -2044,9 +2062,10 @@ __global__ void lr_train_matrix_kernel(const float4* __restrict__ D, int ns, int
 template <int R>
 cudaError_t launch_project_t(const Plan& p, const LowRank& L, const float* alpha, const float* b1,
                              const uint8_t* mask, float* coef, cudaStream_t st) {
-  const int blocks = (p.nv + 127) / 128;
-  lr_project_kernel<R><<<blocks, 128, 0, st>>>(alpha, b1, mask, p.cs, p.phi, L.U, p.nv, p.ntr, (float)p.te_ms,
-                                               (float)(p.tr_ms - p.te_ms), p.inversion ? -1.f : 1.f, coef);
+  const int blocks = (p.nv + kProjThreads - 1) / kProjThreads;
+  auto kernel = b1 != nullptr ? lr_project_kernel<R, true> : lr_project_kernel<R, false>;
+  kernel<<<blocks, kProjThreads, 0, st>>>(alpha, b1, mask, p.cs, p.phi, L.U, p.nv, p.ntr, (float)p.te_ms,
+                                          (float)p.tr_ms, p.inversion ? -1.f : 1.f, coef);
   return cudaGetLastError();
 }
 
