@@ -42,6 +42,13 @@ __device__ __forceinline__ void put_split(__nv_bfloat16* hi, __nv_bfloat16* lo, 
   lo[idx] = __float2bfloat16_rn(v - __bfloat162float(h));
 }
 
+__device__ __forceinline__ void put_split_pair(__nv_bfloat16* hi, __nv_bfloat16* lo, size_t idx, float2 v) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
+  const float2 hf = __bfloat1622float2(h);
+  *reinterpret_cast<__nv_bfloat162*>(hi + idx) = h;
+  *reinterpret_cast<__nv_bfloat162*>(lo + idx) = __floats2bfloat162_rn(v.x - hf.x, v.y - hf.y);
+}
+
 // ---------------------------------------------------------------------------
 // exact linearisation projected onto U: Bloch recursion with tangents (Supporting
 // Information S2), accumulating the sums over the TRs of U[n][r] times the rotated m_y and its
@@ -162,26 +169,33 @@ lr_project_kernel(const float* __restrict__ alpha, const float* __restrict__ b1,
 }
 
 // h_r,j for J.v, written as the K-major split-BF16 operand of the readout GEMM:
-// row r * ny + iy, columns 2 ix (re) and 2 ix + 1 (im)
+// row r * ny + iy, columns 2 ix (re) and 2 ix + 1 (im).  kPrepR basis functions per thread
+// (blockIdx.y): with all R of them a 112 x 88 image filled 39 blocks, each a chain of loads.
+constexpr int kPrepR = 4;
 __global__ void lr_prep_jvp_kernel(const float* __restrict__ v, const float* __restrict__ coef,
                                    const float2* __restrict__ rho, const float* __restrict__ maskf, int nx,
                                    int ny, int nv, int R, __nv_bfloat16* __restrict__ hi,
                                    __nv_bfloat16* __restrict__ lo, int ldk, const int* __restrict__ gate) {
   if (gate != nullptr && *gate == 0) return;
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = blockIdx.x * blockDim.x + threadIdx.x, r0 = blockIdx.y * kPrepR;
   if (j >= nv) return;
   const int iy = j / nx, ix = j - iy * nx;
+  float c[kPrepR], e1[kPrepR], e2[kPrepR];
+#pragma unroll
+  for (int i = 0; i < kPrepR; ++i) {  // R is a multiple of 8
+    c[i] = coef[(size_t)(r0 + i) * nv + j];
+    e1[i] = coef[(size_t)(R + r0 + i) * nv + j];
+    e2[i] = coef[(size_t)(2 * R + r0 + i) * nv + j];
+  }
   const float m = maskf[j];
   const float2 rh = rho[j];
   const float v0 = v[j], v1 = v[nv + j], v2 = v[2 * (size_t)nv + j] * m, v3 = v[3 * (size_t)nv + j] * m;
-  for (int r = 0; r < R; ++r) {
-    const float c = coef[(size_t)r * nv + j];
-    const float t = fmaf(v0, coef[(size_t)(R + r) * nv + j], v1 * coef[(size_t)(2 * R + r) * nv + j]);
+#pragma unroll
+  for (int i = 0; i < kPrepR; ++i) {
+    const float t = fmaf(v0, e1[i], v1 * e2[i]);
     // q = rho t + (v2 + i v3) c ; h = i q
-    const float qr = rh.x * t + v2 * c, qi = rh.y * t + v3 * c;
-    const size_t row = (size_t)(r * ny + iy) * ldk;
-    put_split(hi, lo, row + 2 * ix, -qi);
-    put_split(hi, lo, row + 2 * ix + 1, qr);
+    const float qr = rh.x * t + v2 * c[i], qi = rh.y * t + v3 * c[i];
+    put_split_pair(hi, lo, (size_t)((r0 + i) * ny + iy) * ldk + 2 * ix, make_float2(-qi, qr));
   }
 }
 
@@ -212,23 +226,47 @@ __global__ void lr_transpose_split_kernel(const float* __restrict__ src, int A, 
   }
 }
 
-// s[n][kx] = sum_r U[n][r] H[(r nkx + kx)][ky(n)]   (H rows: ny complex values)
-__global__ void lr_expand_kernel(const float* __restrict__ H, const float* __restrict__ U,
-                                 const int* __restrict__ kyi, int ntr, int nkx, int ny, int R,
-                                 float2* __restrict__ s) {
-  const int kx = blockIdx.x * blockDim.x + threadIdx.x;
-  const int n = blockIdx.y;
-  if (kx >= nkx || n >= ntr) return;
-  const int ky = kyi[n];
+// s[n][kx] = sum_r U[n][r] H[(r nkx + kx)][ky(n)]   (H rows: ny complex values), by
+// phase-encode line: the TRs of a line share its H values, which a thread (kx, ky) holds in
+// registers while it runs over its share of them (blockIdx.z).  Block: 32 kx by kLineKy lines,
+// H through shared memory in whole 32-byte pieces, s written 256 bytes per warp.
+constexpr int kLineKy = 4, kLineSplit = 4;
+template <int R>
+__global__ void __launch_bounds__(32 * kLineKy)
+lr_expand_kernel(const float* __restrict__ H, const float* __restrict__ U, const int* __restrict__ kyptr,
+                 const int* __restrict__ kytr, int nkx, int ny, float2* __restrict__ s) {
+  __shared__ float2 hs[R][32][kLineKy + 1];
+  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 32 + tx;
+  const int kx0 = blockIdx.x * 32, ky0 = blockIdx.y * kLineKy;
   const float2* H2 = reinterpret_cast<const float2*>(H);
-  float sr = 0.f, si = 0.f;
-  for (int r = 0; r < R; ++r) {
-    const float u = __ldg(U + (size_t)n * R + r);
-    const float2 h = H2[((size_t)r * nkx + kx) * ny + ky];
-    sr = fmaf(u, h.x, sr);
-    si = fmaf(u, h.y, si);
+#pragma unroll 8
+  for (int e = tid; e < R * 32 * kLineKy; e += 32 * kLineKy) {
+    const int y = e % kLineKy, x = e / kLineKy % 32, r = e / (32 * kLineKy);
+    const int kx = kx0 + x, ky = ky0 + y;
+    hs[r][x][y] = kx < nkx && ky < ny ? H2[((size_t)r * nkx + kx) * ny + ky] : make_float2(0.f, 0.f);
   }
-  s[(size_t)n * nkx + kx] = make_float2(sr, si);
+  __syncthreads();
+  const int kx = kx0 + tx, ky = ky0 + ty;
+  if (kx >= nkx || ky >= ny) return;
+  float2 h[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) h[r] = hs[r][tx][ty];
+  for (int t = kyptr[ky] + blockIdx.z; t < kyptr[ky + 1]; t += kLineSplit) {
+    const int n = __ldg(kytr + t);
+    const float4* u4 = reinterpret_cast<const float4*>(U + (size_t)n * R);
+    float sr = 0.f, si = 0.f;
+#pragma unroll
+    for (int r = 0; r < R / 4; ++r) {
+      const float4 u = __ldg(u4 + r);
+      const float uv[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        sr = fmaf(uv[i], h[4 * r + i].x, sr);
+        si = fmaf(uv[i], h[4 * r + i].y, si);
+      }
+    }
+    s[(size_t)n * nkx + kx] = make_float2(sr, si);
+  }
 }
 
 // G_r[ky][kx] = sum_r' M_ky[r][r'] H_r'[ky][kx], written as the split operand of the
@@ -259,44 +297,63 @@ __global__ void lr_gram_kernel(const float* __restrict__ H, const float* __restr
   }
 }
 
-// G_r[ky][kx] = sum_{n: ky(n) = ky} U[n][r] w[n][kx] into the same operand layout
-__global__ void lr_gather_kernel(const float2* __restrict__ w, const float* __restrict__ U,
-                                 const int* __restrict__ kyptr, const int* __restrict__ kytr, int nkx, int R,
-                                 __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo, int ldk) {
-  const int ky = blockIdx.x;
-  const int na = kyptr[ky], ne = kyptr[ky + 1];
-  for (int kx = threadIdx.x; kx < nkx; kx += blockDim.x) {
-    float2 g[kMaxRank];
-    for (int r = 0; r < R; ++r) g[r] = make_float2(0.f, 0.f);
-    for (int t = na; t < ne; ++t) {
-      const int n = kytr[t];
-      const float2 wv = w[(size_t)n * nkx + kx];
-      for (int r = 0; r < R; ++r) {
-        const float u = __ldg(U + (size_t)n * R + r);
-        g[r].x = fmaf(u, wv.x, g[r].x);
-        g[r].y = fmaf(u, wv.y, g[r].y);
+// G_r[ky][kx] = sum_{n: ky(n) = ky} U[n][r] w[n][kx] into the same operand layout.  Block:
+// 32 kx by 8 lines, kGatherR basis functions (blockIdx.z); w read 256 bytes per warp, the
+// operand written through shared memory in 32-byte pieces.
+constexpr int kGatherKy = 8, kGatherR = 4;
+__global__ void __launch_bounds__(32 * kGatherKy)
+lr_gather_kernel(const float2* __restrict__ w, const float* __restrict__ U, const int* __restrict__ kyptr,
+                 const int* __restrict__ kytr, int nkx, int ny, int R, __nv_bfloat16* __restrict__ hi,
+                 __nv_bfloat16* __restrict__ lo, int ldk) {
+  __shared__ float2 gs[kGatherR][32][kGatherKy + 1];
+  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 32 + tx;
+  const int kx0 = blockIdx.x * 32, ky0 = blockIdx.y * kGatherKy, r0 = blockIdx.z * kGatherR;
+  const int kx = kx0 + tx, ky = ky0 + ty;
+  float2 g[kGatherR];
+#pragma unroll
+  for (int i = 0; i < kGatherR; ++i) g[i] = make_float2(0.f, 0.f);
+  if (kx < nkx && ky < ny) {
+    const int te = kyptr[ky + 1];
+#pragma unroll 4
+    for (int t = kyptr[ky]; t < te; ++t) {
+      const int n = __ldg(kytr + t);
+      const float2 wv = __ldg(w + (size_t)n * nkx + kx);
+      const float4 u = __ldg(reinterpret_cast<const float4*>(U + (size_t)n * R + r0));  // R a multiple of 8
+      const float uv[kGatherR] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+      for (int i = 0; i < kGatherR; ++i) {
+        g[i].x = fmaf(uv[i], wv.x, g[i].x);
+        g[i].y = fmaf(uv[i], wv.y, g[i].y);
       }
     }
-    for (int r = 0; r < R; ++r) {
-      const size_t row = ((size_t)r * nkx + kx) * ldk;
-      put_split(hi, lo, row + 2 * ky, g[r].x);
-      put_split(hi, lo, row + 2 * ky + 1, g[r].y);
-    }
+  }
+#pragma unroll
+  for (int i = 0; i < kGatherR; ++i) gs[i][tx][ty] = g[i];
+  __syncthreads();
+#pragma unroll
+  for (int e = tid; e < kGatherR * 32 * kGatherKy; e += 32 * kGatherKy) {
+    const int y = e % kGatherKy, x = e / kGatherKy % 32, i = e / (32 * kGatherKy);
+    if (kx0 + x < nkx && ky0 + y < ny)
+      put_split_pair(hi, lo, ((size_t)(r0 + i) * nkx + kx0 + x) * ldk + 2 * (ky0 + y), gs[i][x][y]);
   }
 }
 
-// g_k,j = Re sum_r conj(dh_r,j/dv_k) P_r,j with P rows (r ny + iy), columns 2 ix + re/im
+// Partial sums over one chunk of 8 basis functions (blockIdx.y) of
+//   g_k,j = Re sum_r conj(dh_r,j/dv_k) P_r,j with P rows (r ny + iy), columns 2 ix + re/im
+// into part[chunk][4][nv] (lr_final_sum_kernel adds the chunks).
 __global__ void lr_final_kernel(const float* __restrict__ P, const float* __restrict__ coef,
-                                const float2* __restrict__ rho, const float* __restrict__ maskf, int nx, int ny,
-                                int nv, int R, float* __restrict__ g, const int* __restrict__ gate) {
+                                const float2* __restrict__ rho, int nx, int ny, int nv, int R,
+                                float* __restrict__ part, const int* __restrict__ gate) {
   if (gate != nullptr && *gate == 0) return;
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = blockIdx.x * blockDim.x + threadIdx.x, r0 = blockIdx.y * 8;
   if (j >= nv) return;
   const int iy = j / nx, ix = j - iy * nx;
   const float2* P2 = reinterpret_cast<const float2*>(P);
   float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
   const float2 rh = rho[j];
-  for (int r = 0; r < R; ++r) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {  // R is a multiple of 8
+    const int r = r0 + i;
     const float2 p = P2[(size_t)(r * ny + iy) * nx + ix];
     const float c = coef[(size_t)r * nv + j];
     const float t1 = coef[(size_t)(R + r) * nv + j], t2 = coef[(size_t)(2 * R + r) * nv + j];
@@ -306,11 +363,11 @@ __global__ void lr_final_kernel(const float* __restrict__ P, const float* __rest
     a2 = fmaf(c, p.y, a2);
     a3 = fmaf(-c, p.x, a3);
   }
-  const float m = maskf[j];
-  g[j] = a0 * m;
-  g[nv + j] = a1 * m;
-  g[2 * (size_t)nv + j] = a2 * m;
-  g[3 * (size_t)nv + j] = a3 * m;
+  float* pz = part + (size_t)blockIdx.y * 4 * nv;
+  pz[j] = a0;
+  pz[(size_t)nv + j] = a1;
+  pz[2 * (size_t)nv + j] = a2;
+  pz[3 * (size_t)nv + j] = a3;
 }
 
 // ---------------------------------------------------------------------------
@@ -321,13 +378,6 @@ __global__ void lr_final_kernel(const float* __restrict__ P, const float* __rest
 // reads and writes whole rows; the voxel-order inputs and outputs go through 32 x 32
 // shared-memory tiles.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void put_split_pair(__nv_bfloat16* hi, __nv_bfloat16* lo, size_t idx, float2 v) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
-  const float2 hf = __bfloat1622float2(h);
-  *reinterpret_cast<__nv_bfloat162*>(hi + idx) = h;
-  *reinterpret_cast<__nv_bfloat162*>(lo + idx) = __floats2bfloat162_rn(v.x - hf.x, v.y - hf.y);
-}
-
 // h_r,j = i (rho_j (v0 dc1_r,j + v1 dc2_r,j) + (v2 + i v3) c_r,j) mask_j into rows (ix, r).
 // Block: a 32 x 32 voxel tile and 4 basis functions (blockIdx.z).
 __global__ void __launch_bounds__(256)
@@ -389,11 +439,11 @@ lr_prep_t_kernel(const float* __restrict__ v, const float* __restrict__ coef, co
 // Block (32, 8): 32 consecutive ky (lanes) x 8 image columns; the rows of U of the TRs
 // of its 32 ky values (contiguous in Ug, U gathered in ky order) sit in shared memory,
 // rows padded to R + 1 floats.
-template <int R, bool SPLIT>
+template <int R>
 __global__ void __launch_bounds__(256)
 lr_gram_t_kernel(const float* __restrict__ HT, int ldh, const float* __restrict__ Ug, const int* __restrict__ kyptr,
                  int nx, int ny, __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo, int ldk,
-                 float2* __restrict__ gout, const int* __restrict__ gate) {
+                 const int* __restrict__ gate) {
   if (gate != nullptr && *gate == 0) return;
   extern __shared__ float us[];  // [rows of this ky tile][R + 1]
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 32 + tx;
@@ -431,73 +481,67 @@ lr_gram_t_kernel(const float* __restrict__ HT, int ldh, const float* __restrict_
   }
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    if (SPLIT) put_split_pair(hi, lo, (size_t)(ix * R + r) * ldk + 2 * ky, out[r]);
-    else gout[(size_t)(ix * R + r) * ny + ky] = out[r];
+    put_split_pair(hi, lo, (size_t)(ix * R + r) * ldk + 2 * ky, out[r]);
   }
 }
 
-// The same Gram product when no ky value has more than kGramShort TRs (one TR per fill
-// for up to 8 fills, the usual sequence): the TR-axis sums s_t stay in registers and each
-// output G[(ix, r)][ky] is written as soon as it is formed, so no R-long output array is
-// held (about half the registers of the general kernel, twice the resident warps).
-constexpr int kGramShort = 8;
-
-template <int R, bool SPLIT>
-__global__ void __launch_bounds__(256)
-lr_gram_short_kernel(const float* __restrict__ HT, int ldh, const float* __restrict__ Ug,
-                     const int* __restrict__ kyptr, int nx, int ny, __nv_bfloat16* __restrict__ hi,
-                     __nv_bfloat16* __restrict__ lo, int ldk, float2* __restrict__ gout,
+// The same Gram product when no ky value has more than NS TRs (8, 16 or 32).  Block: 32
+// consecutive ky (lanes) of one image column; warp g takes a quarter of the basis functions,
+// first as inputs (its part of the TR-axis sums s_t of its lane's ky, which the block adds
+// through shared memory), then as outputs.  U by (r, slot, ky) (LowRank::UgS, zero past a ky's
+// TRs): a warp reads it in whole lines from L1 / L2, without a copy in shared memory (rows of
+// U there, in TR order, put the lanes of a warp on two banks when a ky has sixteen TRs).
+// Bound by the latency of its L2 loads: 44 us before at 112 x 88 with 16 fills on 42 blocks of
+// the general kernel, 26 us now.
+constexpr int kGramWarps = 4;
+template <int R, int NS>
+__global__ void __launch_bounds__(32 * kGramWarps)
+lr_gram_short_kernel(const float* __restrict__ HT, int ldh, const float* __restrict__ UgS, int kmax, int nx, int ny,
+                     __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo, int ldk,
                      const int* __restrict__ gate) {
   if (gate != nullptr && *gate == 0) return;
-  extern __shared__ float us[];  // [rows of this ky tile][R + 1]
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 32 + tx;
-  const int ky0 = blockIdx.x * 32;
-  const int t0 = kyptr[ky0], t1 = kyptr[min(ky0 + 32, ny)];
-  for (int e = tid; e < (t1 - t0) * R; e += 256) {
-    const int t = e / R, r = e - t * R;
-    us[t * (R + 1) + r] = Ug[(size_t)t0 * R + e];
+  constexpr int Q = R / kGramWarps;
+  __shared__ float2 part[kGramWarps][NS][32];
+  const int lane = threadIdx.x, g = threadIdx.y, ky = blockIdx.x * 32 + lane, ix = blockIdx.y;
+  const bool in = ky < ny;
+  const float2* H2 = reinterpret_cast<const float2*>(HT) + (size_t)(ix * R + g * Q) * (ldh / 2) + ky;
+  const float* ug = UgS + (size_t)g * Q * kmax * ny + ky;
+  float2 h[Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) h[q] = in ? H2[(size_t)q * (ldh / 2)] : make_float2(0.f, 0.f);
+#pragma unroll 4
+  for (int k = 0; k < NS; ++k) {
+    float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const float u = in && k < kmax ? __ldg(ug + ((size_t)q * kmax + k) * ny) : 0.f;
+      s.x = fmaf(u, h[q].x, s.x);
+      s.y = fmaf(u, h[q].y, s.y);
+    }
+    part[g][k][lane] = s;
   }
   __syncthreads();
-  const int ky = ky0 + tx, ix = blockIdx.y * 8 + ty;
-  if (ky >= ny || ix >= nx) return;
-  const float2* H2 = reinterpret_cast<const float2*>(HT);
-  const int ld2 = ldh / 2;
-  const int ta = kyptr[ky], ns = kyptr[ky + 1] - ta;  // ns <= kGramShort
-  float2 sv[kGramShort];
+  float2 o[Q];
 #pragma unroll
-  for (int k = 0; k < kGramShort; ++k) sv[k] = make_float2(0.f, 0.f);
-  {
-    float2 in[R];
-#pragma unroll
-    for (int q = 0; q < R; ++q) in[q] = H2[(size_t)(ix * R + q) * ld2 + ky];
-#pragma unroll
-    for (int k = 0; k < kGramShort; ++k) {
-      if (k < ns) {
-        const float* un = us + (ta + k - t0) * (R + 1);
-        float sr = 0.f, si = 0.f;
-#pragma unroll
-        for (int q = 0; q < R; ++q) {
-          sr = fmaf(un[q], in[q].x, sr);
-          si = fmaf(un[q], in[q].y, si);
-        }
-        sv[k] = make_float2(sr, si);
-      }
-    }
-  }
+  for (int q = 0; q < Q; ++q) o[q] = make_float2(0.f, 0.f);
 #pragma unroll 4
-  for (int r = 0; r < R; ++r) {
-    float2 o = make_float2(0.f, 0.f);
+  for (int k = 0; k < NS; ++k) {
+    float2 s = part[0][k][lane];
 #pragma unroll
-    for (int k = 0; k < kGramShort; ++k) {
-      if (k < ns) {
-        const float u = us[(ta + k - t0) * (R + 1) + r];
-        o.x = fmaf(u, sv[k].x, o.x);
-        o.y = fmaf(u, sv[k].y, o.y);
-      }
+    for (int i = 1; i < kGramWarps; ++i) {
+      s.x += part[i][k][lane].x;
+      s.y += part[i][k][lane].y;
     }
-    if (SPLIT) put_split_pair(hi, lo, (size_t)(ix * R + r) * ldk + 2 * ky, o);
-    else gout[(size_t)(ix * R + r) * ny + ky] = o;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const float u = in && k < kmax ? __ldg(ug + ((size_t)q * kmax + k) * ny) : 0.f;
+      o[q].x = fmaf(u, s.x, o[q].x);
+      o[q].y = fmaf(u, s.y, o[q].y);
+    }
   }
+  if (!in) return;
+#pragma unroll
+  for (int q = 0; q < Q; ++q) put_split_pair(hi, lo, (size_t)(ix * R + g * Q + q) * ldk + 2 * ky, o[q]);
 }
 
 // ---------------------------------------------------------------------------
@@ -2340,9 +2384,17 @@ static int lr_adjoint_dft_and_final(Plan* p, float* g, const int* gate, cudaStre
     e = launch_tc_gemm(L.op_a4, p->tc[3], L.P, R * ny, 2 * nx, 2 * nkx, 2 * nx, 3, gate, p->dev_err, st);
   }
   if (e == cudaSuccess) {
-    Span sp(p, MRSTAT_K_JHW_DOT, st);
-    lr_final_kernel<<<(p->nv + 255) / 256, 256, 0, st>>>(L.P, L.coef, p->rho, p->maskf, nx, ny, p->nv, R, g, gate);
+    Span sp(p, MRSTAT_K_JHW_DOT, st, 1, 2);  // the chunks' sums and their sum
+    lr_final_kernel<<<dim3((p->nv + 255) / 256, R / 8), 256, 0, st>>>(L.P, L.coef, p->rho, nx, ny, p->nv, R, L.gpart,
+                                                                      gate);
     e = cudaGetLastError();
+    if (e == cudaSuccess) {
+      const int64_t n4 = 4 * (int64_t)p->nv;
+      const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((n4 + kSumThreads - 1) / kSumThreads, kRedBlocks));
+      lr_final_sum_kernel<<<blocks, kSumThreads, 0, st>>>(L.gpart, R / 8, p->maskf, p->nv, 1.f, g, gate, nullptr, p->red,
+                                                          p->ticket, nullptr);
+      e = cudaGetLastError();
+    }
   }
   return e == cudaSuccess ? MRSTAT_OK : cuda_fail(e, "low-rank adjoint DFT");
 }
@@ -2350,7 +2402,7 @@ static int lr_adjoint_dft_and_final(Plan* p, float* g, const int* gate, cudaStre
 static int lr_prep(Plan* p, const float* v, const int* gate, cudaStream_t st) {
   LowRank& L = *p->lr;
   Span sp(p, MRSTAT_K_YCONTRACT, st);
-  lr_prep_jvp_kernel<<<(p->nv + 255) / 256, 256, 0, st>>>(v, L.coef, p->rho, p->maskf, p->nx, p->ny, p->nv, L.R,
+  lr_prep_jvp_kernel<<<dim3((p->nv + 255) / 256, L.R / kPrepR), 256, 0, st>>>(v, L.coef, p->rho, p->maskf, p->nx, p->ny, p->nv, L.R,
                                                           (__nv_bfloat16*)L.a1_hi, (__nv_bfloat16*)L.a1_lo, L.k1,
                                                           gate);
   cudaError_t e = cudaGetLastError();
@@ -2363,8 +2415,10 @@ int lowrank_jvp(Plan* p, const float* v, float2* jv, cudaStream_t st) {
   if (s == MRSTAT_OK) s = lr_forward_dft(p, p->gate, st);
   if (s != MRSTAT_OK) return s;
   Span sp(p, MRSTAT_K_VECTOR, st);
-  dim3 grid((p->nkx + 127) / 128, p->ntr);
-  lr_expand_kernel<<<grid, 128, 0, st>>>(L.H, L.U, p->kyi, p->ntr, p->nkx, p->ny, L.R, jv);
+  const dim3 grid((p->nkx + 31) / 32, (p->ny + kLineKy - 1) / kLineKy, kLineSplit);
+  auto kernel = L.R == 8 ? lr_expand_kernel<8> : L.R == 16 ? lr_expand_kernel<16> : L.R == 24 ? lr_expand_kernel<24>
+                                                                                            : lr_expand_kernel<32>;
+  kernel<<<grid, dim3(32, kLineKy), 0, st>>>(L.H, L.U, L.kyptr, L.kytr, p->nkx, p->ny, jv);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? MRSTAT_OK : cuda_fail(e, "low-rank expand");
 }
@@ -2373,45 +2427,46 @@ int lowrank_jhw(Plan* p, const float2* w, float* g, cudaStream_t st) {
   LowRank& L = *p->lr;
   {
     Span sp(p, MRSTAT_K_VECTOR, st);
-    lr_gather_kernel<<<p->ny, 128, 0, st>>>(w, L.U, L.kyptr, L.kytr, p->nkx, L.R, (__nv_bfloat16*)L.a23_hi,
-                                            (__nv_bfloat16*)L.a23_lo, L.k23);
+    const dim3 grid((p->nkx + 31) / 32, (p->ny + kGatherKy - 1) / kGatherKy, L.R / kGatherR);
+    lr_gather_kernel<<<grid, dim3(32, kGatherKy), 0, st>>>(w, L.U, L.kyptr, L.kytr, p->nkx, p->ny, L.R,
+                                                           (__nv_bfloat16*)L.a23_hi, (__nv_bfloat16*)L.a23_lo, L.k23);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "low-rank gather");
   }
   return lr_adjoint_dft_and_final(p, g, p->gate, st);
 }
 
-// SPLIT: write G as the split-BF16 operand of the adjoint phase-encode GEMM; else as
-// float2 rows [(ix, r)][ky] into gout (the FFT path)
-template <int R, bool SPLIT>
-static cudaError_t launch_gram_t(const Plan& p, const LowRank& L, float2* gout, const int* gate, cudaStream_t st) {
-  const size_t sm = (size_t)L.gram_rows_max * (R + 1) * sizeof(float);
-  const dim3 grid((p.ny + 31) / 32, (p.nx + 7) / 8);
-  __nv_bfloat16* hi = (__nv_bfloat16*)L.a23_hi;
-  __nv_bfloat16* lo = (__nv_bfloat16*)L.a23_lo;
-  if (L.ky_count_max <= kGramShort) {
-    cudaError_t e = cudaFuncSetAttribute(lr_gram_short_kernel<R, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sm);
-    if (e != cudaSuccess) return e;
-    lr_gram_short_kernel<R, SPLIT><<<grid, dim3(32, 8), sm, st>>>(L.H, 2 * p.ny, L.Ug, L.kyptr, p.nx, p.ny, hi, lo,
-                                                                   L.k23, gout, gate);
-  } else {
-    cudaError_t e =
-        cudaFuncSetAttribute(lr_gram_t_kernel<R, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    lr_gram_t_kernel<R, SPLIT><<<grid, dim3(32, 8), sm, st>>>(L.H, 2 * p.ny, L.Ug, L.kyptr, p.nx, p.ny, hi, lo, L.k23,
-                                                               gout, gate);
-  }
+template <int R, int NS>
+static cudaError_t launch_gram_short(const Plan& p, const LowRank& L, const int* gate, cudaStream_t st) {
+  const dim3 grid((p.ny + 31) / 32, p.nx);
+  lr_gram_short_kernel<R, NS><<<grid, dim3(32, kGramWarps), 0, st>>>(L.H, 2 * p.ny, L.UgS, L.ky_count_max, p.nx, p.ny,
+                                                                 (__nv_bfloat16*)L.a23_hi, (__nv_bfloat16*)L.a23_lo,
+                                                                 L.k23, gate);
   return cudaGetLastError();
 }
 
-template <bool SPLIT>
-static cudaError_t launch_gram(const Plan& p, const LowRank& L, float2* gout, const int* gate, cudaStream_t st) {
+// The Gram product written as the split-BF16 operand of the adjoint phase-encode GEMM: the
+// register form for up to 32 TRs per ky, the general one beyond.
+template <int R>
+static cudaError_t launch_gram_t(const Plan& p, const LowRank& L, const int* gate, cudaStream_t st) {
+  if (L.ky_count_max <= 8) return launch_gram_short<R, 8>(p, L, gate, st);
+  if (L.ky_count_max <= 16) return launch_gram_short<R, 16>(p, L, gate, st);
+  if (L.ky_count_max <= 32) return launch_gram_short<R, 32>(p, L, gate, st);
+  const size_t sm = (size_t)L.gram_rows_max * (R + 1) * sizeof(float);
+  const dim3 grid((p.ny + 31) / 32, (p.nx + 7) / 8);
+  cudaError_t e = cudaFuncSetAttribute(lr_gram_t_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  lr_gram_t_kernel<R><<<grid, dim3(32, 8), sm, st>>>(L.H, 2 * p.ny, L.Ug, L.kyptr, p.nx, p.ny, (__nv_bfloat16*)L.a23_hi,
+                                                     (__nv_bfloat16*)L.a23_lo, L.k23, gate);
+  return cudaGetLastError();
+}
+
+static cudaError_t launch_gram(const Plan& p, const LowRank& L, const int* gate, cudaStream_t st) {
   switch (L.R) {
-    case 8: return launch_gram_t<8, SPLIT>(p, L, gout, gate, st);
-    case 16: return launch_gram_t<16, SPLIT>(p, L, gout, gate, st);
-    case 24: return launch_gram_t<24, SPLIT>(p, L, gout, gate, st);
-    default: return launch_gram_t<32, SPLIT>(p, L, gout, gate, st);
+    case 8: return launch_gram_t<8>(p, L, gate, st);
+    case 16: return launch_gram_t<16>(p, L, gate, st);
+    case 24: return launch_gram_t<24>(p, L, gate, st);
+    default: return launch_gram_t<32>(p, L, gate, st);
   }
 }
 
@@ -2436,7 +2491,7 @@ static int lowrank_jhjv_full_readout(Plan* p, const float* v, float* out, double
   }
   if (e == cudaSuccess) {
     Span sp(p, MRSTAT_K_VECTOR, st);
-    e = launch_gram<true>(*p, L, nullptr, gate, st);
+    e = launch_gram(*p, L, gate, st);
   }
   if (e == cudaSuccess) {
     Span sp(p, MRSTAT_K_XDFT_ADJ, st);
