@@ -246,6 +246,7 @@ int lowrank_setup(Plan* p, const float* U_dev, int R, cudaStream_t st);
 void lowrank_free(LowRank* L);
 cudaError_t lowrank_project(const Plan& p, const LowRank& L, const float* alpha, const float* b1,
                             const uint8_t* mask, float* coef, cudaStream_t st);
+cudaError_t lowrank_adopt(Plan* p, const float* coef, cudaStream_t st);
 int lowrank_jvp(Plan* p, const float* v, float2* jv, cudaStream_t st);
 int lowrank_jhw(Plan* p, const float2* w, float* g, cudaStream_t st);
 // Re(J^H J) v; with vdot also *vdot = <v, Re(J^H J) v>, with vv also *vv = <v, v> (fused

@@ -690,20 +690,33 @@ __device__ __forceinline__ void fft16(float2 (&a)[16]) {
 __host__ __device__ constexpr int col_row(int ny) { return 17 * (ny / 16); }
 
 // coefT[(k R + r)][ix][iy] = coef[(k R + r)][iy nx + ix]: the coefficients in image-column
-// order, so that a block working on one column ix reads them contiguously (32 x 32 tiles)
-__global__ void lr_coef_transpose_kernel(const float* __restrict__ coef, int nx, int ny, float* __restrict__ coefT) {
+// order, so that a block working on one column ix reads them contiguously (32 x 32 tiles).
+// With copy, the tile also goes there in the order it was read (a caller's coefficients are
+// adopted and put in column order in one pass over them).
+__global__ void lr_coef_transpose_kernel(const float* __restrict__ coef, int nx, int ny, float* __restrict__ coefT,
+                                         float* __restrict__ copy) {
   __shared__ float tile[32][33];
   const int plane = blockIdx.z;
   const int ix0 = blockIdx.x * 32, iy0 = blockIdx.y * 32;
   const size_t nv = (size_t)nx * ny;
   const float* src = coef + plane * nv;
   float* dst = coefT + plane * nv;
-  for (int k = threadIdx.y; k < 32; k += 8) {
-    const int iy = iy0 + k, ix = ix0 + threadIdx.x;
-    tile[k][threadIdx.x] = (iy < ny && ix < nx) ? src[(size_t)iy * nx + ix] : 0.f;
+  float v[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int iy = iy0 + threadIdx.y + 8 * i, ix = ix0 + threadIdx.x;
+    v[i] = (iy < ny && ix < nx) ? src[(size_t)iy * nx + ix] : 0.f;
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int k = threadIdx.y + 8 * i, iy = iy0 + k, ix = ix0 + threadIdx.x;
+    tile[k][threadIdx.x] = v[i];
+    if (copy != nullptr && iy < ny && ix < nx) copy[plane * nv + (size_t)iy * nx + ix] = v[i];
   }
   __syncthreads();
-  for (int k = threadIdx.y; k < 32; k += 8) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int k = threadIdx.y + 8 * i;
     const int ix = ix0 + k, iy = iy0 + threadIdx.x;
     if (ix < nx && iy < ny) dst[(size_t)ix * ny + iy] = tile[threadIdx.x][k];
   }
@@ -2520,7 +2533,22 @@ static cudaError_t ensure_coef_columns(Plan* p, cudaStream_t st) {
   LowRank& L = *p->lr;
   if (!L.coefT_dirty && L.coefT_src == L.coef) return cudaSuccess;
   const dim3 grid((p->nx + 31) / 32, (p->ny + 31) / 32, 3 * L.R);
-  lr_coef_transpose_kernel<<<grid, dim3(32, 8), 0, st>>>(L.coef, p->nx, p->ny, L.coefT);
+  lr_coef_transpose_kernel<<<grid, dim3(32, 8), 0, st>>>(L.coef, p->nx, p->ny, L.coefT, nullptr);
+  L.coefT_src = L.coef;
+  L.coefT_dirty = false;
+  return cudaGetLastError();
+}
+
+// Adopts a caller's coefficients: into L.coef and, where the column kernels read them, in
+// image-column order in the same pass.
+cudaError_t lowrank_adopt(Plan* p, const float* coef, cudaStream_t st) {
+  LowRank& L = *p->lr;
+  if (!L.column_path) {
+    L.coefT_dirty = true;
+    return cudaMemcpyAsync(L.coef, coef, (size_t)3 * L.R * p->nv * sizeof(float), cudaMemcpyDeviceToDevice, st);
+  }
+  const dim3 grid((p->nx + 31) / 32, (p->ny + 31) / 32, 3 * L.R);
+  lr_coef_transpose_kernel<<<grid, dim3(32, 8), 0, st>>>(coef, p->nx, p->ny, L.coefT, L.coef);
   L.coefT_src = L.coef;
   L.coefT_dirty = false;
   return cudaGetLastError();

@@ -104,11 +104,11 @@ int mrstat_lowrank_linearize(mrstat_plan* plan_, const float* alpha, const float
   if (coef == nullptr) {
     Span sp(p, MRSTAT_K_BLOCH, st);
     e = lowrank_project(*p, L, alpha, b1, mask, L.coef, st);
+    L.coefT_dirty = true;
   } else {
-    e = cudaMemcpyAsync(L.coef, coef, (size_t)3 * L.R * p->nv * sizeof(float), cudaMemcpyDeviceToDevice, st);
+    e = lowrank_adopt(p, coef, st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "low-rank coefficients");
-  L.coefT_dirty = true;
   L.active = true;
   p->linearized = true;
   return MRSTAT_OK;
