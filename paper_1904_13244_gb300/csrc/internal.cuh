@@ -28,8 +28,8 @@ constexpr int kRedSlots = 16 * kRedBlocks;
 // every seg-th TR, column-major.
 struct RxLin {
   float* fac = nullptr;  // [6][nx][nys]
-  float* st = nullptr;   // [nseg][ns][nx][nys]
-  int seg = 0, nseg = 0, ns = 6;
+  float* st = nullptr;   // [cap][ns][nx][nys], nseg of them in use
+  int seg = 0, nseg = 0, cap = 0, ns = 6;
 };
 
 struct Plan {

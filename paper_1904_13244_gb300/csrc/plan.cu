@@ -95,17 +95,18 @@ cudaError_t ensure_rx(Plan* p, RxLin* L, int ns, int seg) {
   const int nseg = (p->ntr + seg - 1) / seg;
   cudaError_t e = cudaSuccess;
   if (L->fac == nullptr) e = dalloc(p, &L->fac, 6 * nvp);
-  if (e == cudaSuccess && L->st != nullptr && L->nseg < nseg) {
+  if (e == cudaSuccess && L->st != nullptr && L->cap < nseg) {
     e = cudaDeviceSynchronize();
     cudaFree(L->st);
-    p->bytes -= (int64_t)((size_t)L->nseg * L->ns * nvp * sizeof(float));
+    p->bytes -= (int64_t)((size_t)L->cap * L->ns * nvp * sizeof(float));
     L->st = nullptr;
   }
   if (e == cudaSuccess && L->st == nullptr) {
     e = dalloc(p, &L->st, (size_t)nseg * ns * nvp);
     L->ns = ns;
-    L->nseg = nseg;
+    L->cap = nseg;
   }
+  L->nseg = nseg;
   return e;
 }
 
@@ -825,7 +826,6 @@ int mrstat_forward_ckpt(mrstat_plan* plan, const float* alpha, const float* b1, 
     if (e == cudaSuccess && plan->rxc_maskf == nullptr) e = dalloc(plan, &plan->rxc_maskf, (size_t)plan->nv);
     if (e != cudaSuccess) return cuda_fail(e, "checkpoint allocation");
     plan->rxc.seg = seg;
-    plan->rxc.nseg = (plan->ntr + seg - 1) / seg;
     {
       Span sp(plan, MRSTAT_K_BLOCH, st);
       e = launch_rx_states(*plan, plan->rxc, alpha, mask, plan->rxc_rho, plan->rxc_maskf, st);
