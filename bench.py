@@ -816,9 +816,10 @@ def main():
     # the plain FP32 form on the same inputs, for the comparison the metric asks for
     plain = None
     if args.form not in ("plain", "recompute"):
-        # the plain FP32 form in both variants, cached time courses and the recompute form
-        # (the recursion re-run inside every product from states every `segment` TRs); the
-        # faster one is the plain form the comparison uses
+        # the plain FP32 form in both variants, the plan's own (key "stored": the recursion
+        # re-run in packed pairs; time courses are stored only where that does not apply) and
+        # mrstat_set_recompute's (states every `segment` TRs); the faster one is the plain form
+        # the comparison uses
         pplan = mr.Plan(seq)
         nst = max(1, args.steps // 4)
         pms, pstats, _ = timed(pplan, make_step(pplan, "plain"), nst, all_kernels)
@@ -902,9 +903,9 @@ def main():
         ev1.record(stream)
         torch.cuda.synchronize()
         lin_ms = ev0.elapsed_time(ev1) / reps
-        # per voxel, TR and isochromat: the pulse applied to m and both tangents (3 x 15
-        # flops) and two relaxations with the tangents' source terms (2 x 25 flops)
-        flops = seq.nv * seq.ntr * 32 * 95.0
+        # per voxel, TR and mirrored pair of isochromats: the pulse applied to m and both
+        # tangents (3 x 15 flops) and one relaxation with the tangents' source terms (26)
+        flops = seq.nv * seq.ntr * 16 * 71.0
         fp32_peak = torch.cuda.get_device_properties(0).multi_processor_count * 128 * 2 * 2.07e9
         sms, _, _ = timed(sp_plan, make_step(sp_plan, "plain"), max(3, args.steps // 6), ())
         slice_prof = {"linearize_ms": lin_ms, "isochromats": 32, "rf_substeps": 16,
@@ -1024,6 +1025,10 @@ def main():
         # v and the phase 15, the adjoint phase and the four tangent products 17, the block
         # sums 2)
         work = {"jhw_dot": (86.0 * nv * ntr, "alu")}
+    elif full_readout and ny <= 256:
+        # one launch per product re-running the recursion: 41 multiply-adds (or half of one)
+        # per voxel-TR; the linearisation 21
+        work = {"jhw_dot": (2 * 41.0 * nv * ntr, "alu"), "bloch": (2 * 21.0 * nv * ntr, "alu")}
     else:
         work = {"jhw_dot": (d_bytes + ntr_pad * nx * 8 + nv * (8 + 4 + 16) + ntr_pad * 4, "hbm"),
                 "ycontract": (d_bytes + nv * 24 + ntr * nx * 8 + ntr_pad * 4, "hbm"),
@@ -1078,6 +1083,8 @@ def main():
            "xdft_adj": "tc_gemm.cu", "mlp_infer": "mlp.cu"}
     if lowrank_like:
         src.update({"jhw_dot": "lowrank.cu", "ycontract": "lowrank.cu"})
+    if args.form in ("plain", "split") and ny <= 256:
+        src.update({"jhw_dot": "recur.cu", "ycontract": "recur.cu", "bloch": "recur.cu"})
     if args.form == "recompute":
         src.update({"jhw_dot": "fused.cu"})
     if dom == "mlp_infer":
@@ -1097,7 +1104,7 @@ def main():
     recon = None
     if not args.no_recon and rank == 0:
         if args.form == "recompute":
-            plan.set_recompute(0)  # the Gauss-Newton solve keeps cached time courses
+            plan.set_recompute(0)  # the Gauss-Newton solve runs in the plan's own form
         truth = torch.tensor(alpha_h, device="cuda")
         d, noise = noisy_data(torch, plan, truth, None)
         runs = [("plain", dict(hessian=0)), ("lowrank", dict(hessian=1))]
@@ -1193,10 +1200,10 @@ def main():
         form_desc = {"surrogate": f"learned surrogate + low-rank form (rank {R} time basis, MLP {args.hidden}x3 "
                                   f"tcgen05 coefficients, {dft}, per-ky Gram J^H J v)",
                      "lowrank": f"low-rank form (rank {R} time basis, {dft}, per-ky Gram J^H J v)",
-                     "plain": "plain FP32 form (cached time courses, FP32 readout DFT)",
+                     "plain": "plain FP32 form (recursion re-run in every product, FP32 readout DFT)",
                      "recompute": f"plain FP32 form, recompute variant (Bloch recursion re-run in every product "
                                   f"from states every {args.segment} TRs, fused with the phase-encode sums)",
-                     "split": "split-BF16 form (cached time courses, tcgen05 readout DFT)"}[args.form]
+                     "split": "split-BF16 form (recursion re-run in every product, tcgen05 readout DFT)"}[args.form]
         l2 = ("inputs larger than L2 (cached time courses %.0f MB)" % (d_bytes / 1e6) if not lowrank_like
               else "L2 not flushed: the low-rank operands (~%.0f MB) are L2-resident by design; the "
                    "linearisation streams the parameters and writes the coefficients each step"
