@@ -2361,7 +2361,7 @@ static int lr_forward_dft(Plan* p, const int* gate, cudaStream_t st) {
   cudaError_t e;
   {
     Span sp(p, MRSTAT_K_XDFT, st);
-    e = launch_tc_gemm(L.op_a1, p->tc[1], L.X1, R * ny, 2 * nkx, 2 * nx, 2 * nkx, 3, gate, p->dev_err, st);
+    e = launch_tc_gemm(L.op_a1, p->tc[1], L.X1, R * ny, 2 * nkx, 2 * nx, 2 * nkx, gate, p->dev_err, st);
   }
   if (e == cudaSuccess) {
     Span sp(p, MRSTAT_K_VECTOR, st);
@@ -2372,7 +2372,7 @@ static int lr_forward_dft(Plan* p, const int* gate, cudaStream_t st) {
   }
   if (e == cudaSuccess) {
     Span sp(p, MRSTAT_K_XDFT, st);
-    e = launch_tc_gemm(L.op_a23, L.op_by, L.H, R * nkx, 2 * ny, 2 * ny, 2 * ny, 3, gate, p->dev_err, st);
+    e = launch_tc_gemm(L.op_a23, L.op_by, L.H, R * nkx, 2 * ny, 2 * ny, 2 * ny, gate, p->dev_err, st);
   }
   return e == cudaSuccess ? MRSTAT_OK : cuda_fail(e, "low-rank DFT");
 }
@@ -2383,7 +2383,7 @@ static int lr_adjoint_dft_and_final(Plan* p, float* g, const int* gate, cudaStre
   cudaError_t e;
   {
     Span sp(p, MRSTAT_K_XDFT_ADJ, st);
-    e = launch_tc_gemm(L.op_a23, L.op_bya, L.Y3, R * nkx, 2 * ny, 2 * ny, 2 * ny, 3, gate, p->dev_err, st);
+    e = launch_tc_gemm(L.op_a23, L.op_bya, L.Y3, R * nkx, 2 * ny, 2 * ny, 2 * ny, gate, p->dev_err, st);
   }
   if (e == cudaSuccess) {
     Span sp(p, MRSTAT_K_VECTOR, st);
@@ -2394,7 +2394,7 @@ static int lr_adjoint_dft_and_final(Plan* p, float* g, const int* gate, cudaStre
   }
   if (e == cudaSuccess) {
     Span sp(p, MRSTAT_K_XDFT_ADJ, st);
-    e = launch_tc_gemm(L.op_a4, p->tc[3], L.P, R * ny, 2 * nx, 2 * nkx, 2 * nx, 3, gate, p->dev_err, st);
+    e = launch_tc_gemm(L.op_a4, p->tc[3], L.P, R * ny, 2 * nx, 2 * nkx, 2 * nx, gate, p->dev_err, st);
   }
   if (e == cudaSuccess) {
     Span sp(p, MRSTAT_K_JHW_DOT, st, 1, 2);  // the chunks' sums and their sum
@@ -2500,7 +2500,7 @@ static int lowrank_jhjv_full_readout(Plan* p, const float* v, float* out, double
   }
   if (e == cudaSuccess) {
     Span sp(p, MRSTAT_K_XDFT, st);
-    e = launch_tc_gemm(L.op_a23, L.op_by, L.H, R * nx, 2 * ny, 2 * ny, 2 * ny, 3, gate, p->dev_err, st);
+    e = launch_tc_gemm(L.op_a23, L.op_by, L.H, R * nx, 2 * ny, 2 * ny, 2 * ny, gate, p->dev_err, st);
   }
   if (e == cudaSuccess) {
     Span sp(p, MRSTAT_K_VECTOR, st);
@@ -2508,7 +2508,7 @@ static int lowrank_jhjv_full_readout(Plan* p, const float* v, float* out, double
   }
   if (e == cudaSuccess) {
     Span sp(p, MRSTAT_K_XDFT_ADJ, st);
-    e = launch_tc_gemm(L.op_a23, L.op_bya, L.Y3, R * nx, 2 * ny, 2 * ny, 2 * ny, 3, gate, p->dev_err, st);
+    e = launch_tc_gemm(L.op_a23, L.op_bya, L.Y3, R * nx, 2 * ny, 2 * ny, 2 * ny, gate, p->dev_err, st);
   }
   if (e == cudaSuccess) {
     Span sp(p, MRSTAT_K_JHW_DOT, st);

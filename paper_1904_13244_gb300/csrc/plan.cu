@@ -278,7 +278,7 @@ int do_xdft(Plan* p, const float2* A, float2* out, const int* gate, cudaStream_t
     if (e != cudaSuccess) return cuda_fail(e, "split launch");
     Span sp(p, MRSTAT_K_XDFT, st);
     e = launch_tc_gemm(p->tc[0], p->tc[1], reinterpret_cast<float*>(out), p->ntr, 2 * p->nkx, 2 * p->nx,
-                       2 * p->nkx, 3, gate, p->dev_err, st);
+                       2 * p->nkx, gate, p->dev_err, st);
   } else {
     Span sp(p, MRSTAT_K_XDFT, st);
     e = launch_cgemm(A, p->ft, out, p->ntr, p->nkx, p->nx, gate, st);
@@ -297,7 +297,7 @@ int do_xdft_adj(Plan* p, const float2* w, float2* out, const int* gate, cudaStre
     if (e != cudaSuccess) return cuda_fail(e, "split launch");
     Span sp(p, MRSTAT_K_XDFT_ADJ, st);
     e = launch_tc_gemm(p->tc[2], p->tc[3], reinterpret_cast<float*>(out), p->ntr, 2 * p->nx, 2 * p->nkx,
-                       2 * p->nx, 3, gate, p->dev_err, st);
+                       2 * p->nx, gate, p->dev_err, st);
   } else {
     Span sp(p, MRSTAT_K_XDFT_ADJ, st);
     e = launch_cgemm(w, p->fh, out, p->ntr, p->nx, p->nkx, gate, st);

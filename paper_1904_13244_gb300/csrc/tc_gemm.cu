@@ -42,7 +42,7 @@ template <int BN, int STAGES>
 __global__ void __launch_bounds__(128, 2)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap ta_hi, const __grid_constant__ CUtensorMap ta_lo,
                const __grid_constant__ CUtensorMap tb_hi, const __grid_constant__ CUtensorMap tb_lo,
-               float* __restrict__ C, int M, int N, int K, int ldc, int nprod, const int* __restrict__ gate,
+               float* __restrict__ C, int M, int N, int K, int ldc, const int* __restrict__ gate,
                int* __restrict__ err) {
   using TS = TileShape<BN, STAGES>;
   static_assert(BN == 64 || BN == 128, "N tiles of 64 or 128 columns");
@@ -85,13 +85,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap ta_hi, const __grid_constant_
       uint8_t* a_lo = a_hi + TS::kA;
       uint8_t* b_hi = a_lo + TS::kA;
       uint8_t* b_lo = b_hi + TS::kB;
-      mbar_expect_tx(&full[s], nprod == 3 ? TS::kStage : TS::kA + TS::kB);
+      mbar_expect_tx(&full[s], TS::kStage);
       tma_load_2d(&ta_hi, &full[s], a_hi, c * BK, m0);
       tma_load_2d(&tb_hi, &full[s], b_hi, c * BK, n0);
-      if (nprod == 3) {
-        tma_load_2d(&ta_lo, &full[s], a_lo, c * BK, m0);
-        tma_load_2d(&tb_lo, &full[s], b_lo, c * BK, n0);
-      }
+      tma_load_2d(&ta_lo, &full[s], a_lo, c * BK, m0);
+      tma_load_2d(&tb_lo, &full[s], b_lo, c * BK, n0);
       issued = c + 1;
     }
   } else if (warp == 1 && lane == 0) {
@@ -111,10 +109,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap ta_hi, const __grid_constant_
       for (int k = 0; k < BK / 16; ++k) {
         const uint64_t off = 2ull * k;  // 16 BF16 = 32 B along K, in 16-byte units
         mma_bf16(tmem, dah + off, dbh + off, idesc, (c > 0 || k > 0) ? 1u : 0u);
-        if (nprod == 3) {
-          mma_bf16(tmem, dah + off, dbl + off, idesc, 1u);
-          mma_bf16(tmem, dal + off, dbh + off, idesc, 1u);
-        }
+        mma_bf16(tmem, dah + off, dbl + off, idesc, 1u);
+        mma_bf16(tmem, dal + off, dbh + off, idesc, 1u);
       }
       mma_commit(&empty[s]);
     }
@@ -188,7 +184,7 @@ template <int BN, int STAGES>
 __global__ void __launch_bounds__(192, 1)
 tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap ta_hi, const __grid_constant__ CUtensorMap ta_lo,
                           const __grid_constant__ CUtensorMap tb_hi, const __grid_constant__ CUtensorMap tb_lo,
-                          float* __restrict__ C, int M, int N, int K, int ldc, int nprod,
+                          float* __restrict__ C, int M, int N, int K, int ldc,
                           const int* __restrict__ gate, int* __restrict__ err) {
   using PS = PersistentShape<BN, STAGES>;
   static_assert(BN == 64 || BN == 128, "N tiles of 64 or 128 columns");
@@ -244,13 +240,11 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap ta_hi, const __gri
           uint8_t* a_lo = a_hi + PS::kA;
           uint8_t* b_hi = a_lo + PS::kA;
           uint8_t* b_lo = b_hi + PS::kB;
-          mbar_expect_tx(&full[s], nprod == 3 ? PS::kStage : PS::kA + PS::kB);
+          mbar_expect_tx(&full[s], PS::kStage);
           tma_load_2d(&ta_hi, &full[s], a_hi, c * BK, m0);
           tma_load_2d(&tb_hi, &full[s], b_hi, c * BK, n0);
-          if (nprod == 3) {
-            tma_load_2d(&ta_lo, &full[s], a_lo, c * BK, m0);
-            tma_load_2d(&tb_lo, &full[s], b_lo, c * BK, n0);
-          }
+          tma_load_2d(&ta_lo, &full[s], a_lo, c * BK, m0);
+          tma_load_2d(&tb_lo, &full[s], b_lo, c * BK, n0);
           issued = g + 1;
         }
       }
@@ -282,10 +276,8 @@ tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap ta_hi, const __gri
           for (int k = 0; k < BK / 16; ++k) {
             const uint64_t off = 2ull * k;
             mma_bf16(d, dah + off, dbh + off, idesc, (c > 0 || k > 0) ? 1u : 0u);
-            if (nprod == 3) {
-              mma_bf16(d, dah + off, dbl + off, idesc, 1u);
-              mma_bf16(d, dal + off, dbh + off, idesc, 1u);
-            }
+            mma_bf16(d, dah + off, dbl + off, idesc, 1u);
+            mma_bf16(d, dal + off, dbh + off, idesc, 1u);
           }
           mma_commit(&empty[s]);
         }
@@ -416,14 +408,14 @@ void tc_gemm_set_persistent(bool on) { g_tc_persistent = on; }
 
 template <int BN, int STAGES>
 static cudaError_t launch_tile(const TcOperand& a, const TcOperand& b, float* C, int M, int N, int K, int ldc,
-                               int nprod, const int* gate, int* err, cudaStream_t st) {
+                               const int* gate, int* err, cudaStream_t st) {
   const size_t sm = TileShape<BN, STAGES>::kSmem;
   // the attribute is per device; setting it on every launch is cheap
   cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<BN, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sm);
   if (e != cudaSuccess) return e;
   dim3 grid((M + BM - 1) / BM, (N + BN - 1) / BN);
-  tc_gemm_kernel<BN, STAGES><<<grid, 128, sm, st>>>(a.hi, a.lo, b.hi, b.lo, C, M, N, K, ldc, nprod, gate, err);
+  tc_gemm_kernel<BN, STAGES><<<grid, 128, sm, st>>>(a.hi, a.lo, b.hi, b.lo, C, M, N, K, ldc, gate, err);
   return cudaGetLastError();
 }
 
@@ -433,7 +425,7 @@ static cudaError_t launch_tile(const TcOperand& a, const TcOperand& b, float* C,
 // 128-wide tiles use 3 stages (about 190 KB of shared memory, one CTA per SM).
 template <int BN, int STAGES>
 static cudaError_t launch_persistent(const TcOperand& a, const TcOperand& b, float* C, int M, int N, int K,
-                                     int ldc, int nprod, const int* gate, int* err, cudaStream_t st) {
+                                     int ldc, const int* gate, int* err, cudaStream_t st) {
   const size_t sm = PersistentShape<BN, STAGES>::kSmem;
   cudaError_t e = cudaFuncSetAttribute(tc_gemm_persistent_kernel<BN, STAGES>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -443,25 +435,25 @@ static cudaError_t launch_persistent(const TcOperand& a, const TcOperand& b, flo
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
   const int grid = std::max(1, std::min(tiles, sms));
-  tc_gemm_persistent_kernel<BN, STAGES><<<grid, 192, sm, st>>>(a.hi, a.lo, b.hi, b.lo, C, M, N, K, ldc, nprod,
+  tc_gemm_persistent_kernel<BN, STAGES><<<grid, 192, sm, st>>>(a.hi, a.lo, b.hi, b.lo, C, M, N, K, ldc,
                                                                gate, err);
   return cudaGetLastError();
 }
 
 cudaError_t launch_tc_gemm(const TcOperand& a, const TcOperand& b, float* C, int M, int N, int K, int ldc,
-                           int nprod, const int* gate, int* err, cudaStream_t st) {
+                           const int* gate, int* err, cudaStream_t st) {
   if (M == 0 || N == 0) return cudaSuccess;
   if (a.box != BM) return cudaErrorInvalidValue;
   if (g_tc_persistent) {
-    if (b.box == 128) return launch_persistent<128, 3>(a, b, C, M, N, K, ldc, nprod, gate, err, st);
-    if (b.box == 64) return launch_persistent<64, 4>(a, b, C, M, N, K, ldc, nprod, gate, err, st);
+    if (b.box == 128) return launch_persistent<128, 3>(a, b, C, M, N, K, ldc, gate, err, st);
+    if (b.box == 64) return launch_persistent<64, 4>(a, b, C, M, N, K, ldc, gate, err, st);
     return cudaErrorInvalidValue;
   }
   switch (b.box) {
     case 64:
-      if ((K + BK - 1) / BK <= 8) return launch_tile<64, 2>(a, b, C, M, N, K, ldc, nprod, gate, err, st);
-      return launch_tile<64, 4>(a, b, C, M, N, K, ldc, nprod, gate, err, st);
-    case 128: return launch_tile<128, 3>(a, b, C, M, N, K, ldc, nprod, gate, err, st);
+      if ((K + BK - 1) / BK <= 8) return launch_tile<64, 2>(a, b, C, M, N, K, ldc, gate, err, st);
+      return launch_tile<64, 4>(a, b, C, M, N, K, ldc, gate, err, st);
+    case 128: return launch_tile<128, 3>(a, b, C, M, N, K, ldc, gate, err, st);
     default: return cudaErrorInvalidValue;
   }
 }
