@@ -76,6 +76,9 @@ bloch_slice_kernel(const float* __restrict__ alpha, const uint8_t* __restrict__ 
       t1 = expf(alpha[j]);
       t2 = expf(alpha[nv + j]);
     }
+    // a voxel outside the mask stands for zeros whatever its parameters are (NaN too)
+    t1 = on ? t1 : 1000.f;
+    t2 = on ? t2 : 100.f;
     const float x1s = expm1f(-tr / t1), x2s = expm1f(-tr / t2);
     x1[w] = pk::both(x1s);
     x2[w] = pk::both(x2s);

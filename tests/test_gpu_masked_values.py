@@ -1,0 +1,78 @@
+"""Parameters outside the mask do not count, whatever they hold: NaN, or the -inf that the log
+of a map leaves where the map is zero.  Every output is bit for bit the one with finite
+parameters there.  The masks leave warps and blocks partly and wholly empty.
+"""
+import numpy as np
+import pytest
+
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+BAD = [float("nan"), float("-inf")]
+
+
+def make(nx, ny, fills, extra=0, npar=4):
+    rng = np.random.default_rng([nx, ny])
+    seq = synth.make_sequence(nx, ny, fills, 7.8, 3.4, seed=nx, extra_trs=extra)
+    nv = seq.nv
+    alpha = [rng.uniform(np.log(200), np.log(3000), nv), rng.uniform(np.log(20), np.log(300), nv),
+             rng.uniform(0.5, 1, nv), rng.uniform(-1, 1, nv), rng.uniform(0.8, 1.2, nv)][:npar]
+    mask = (rng.random(nv) < 0.7).astype(np.uint8)
+    mask[nv // 3: nv // 3 + nv // 4] = 0
+    mask[-1], mask[0] = 0, 1
+    dev = lambda a, t=torch.float32: torch.tensor(np.ascontiguousarray(a), dtype=t, device="cuda")  # noqa: E731
+    v = rng.standard_normal((npar, nv))
+    return (seq, dev(np.stack(alpha)), dev(mask, torch.uint8), dev(v),
+            dev(synth.random_kspace(seq.ntr, seq.nkx, 2), torch.complex64))
+
+
+def spoil(x, mask, value, rows=slice(None)):
+    x = x.clone()
+    x[rows, mask == 0] = value
+    return x
+
+
+def all_equal(got, ref):
+    return all(bool(torch.isfinite(torch.view_as_real(r) if r.is_complex() else r).all()) for r in ref) and \
+        all(torch.equal(g, r) for g, r in zip(got, ref))
+
+
+def exact_calls(plan, a, mask, v, w, b1=None):
+    plan.linearize(a, b1=b1, mask=mask)
+    out = [plan.jvp(v), plan.jhw(w), plan.jhjv(v), plan.forward(a, b1=b1, mask=mask)]
+    return out + [plan.timecourses(c) for c in range(a.shape[0] - 1)]
+
+
+# 13 x 9: a lane per voxel in the forward kernel; 144 x 136: four of them
+@pytest.mark.parametrize("value", BAD)
+@pytest.mark.parametrize("nx,ny,fills", [(13, 9, 3), (144, 136, 1)])
+@pytest.mark.parametrize("n_iso", [1, 8, 32])
+def test_slice_profile_relaxation_times(n_iso, nx, ny, fills, value):
+    import paper_1904_13244_gb300 as mr
+    seq, a, mask, v, w = make(nx, ny, fills, extra=2)
+    bad = spoil(a, mask, value, slice(0, 2))
+    with mr.Plan(seq) as plan:
+        plan.set_slice_profile(n_iso, 6, 0.2, 4.0, 2.0)
+        ref = exact_calls(plan, a, mask, v, w)
+        got = exact_calls(plan, bad, mask, v, w)
+    assert all_equal(got, ref)
+    assert not any(t[:, mask == 0].any() for t in got[4:])
+
+
+@pytest.mark.parametrize("value", BAD)
+def test_slice_profile_solve(value):
+    import paper_1904_13244_gb300 as mr
+    seq, a, mask, _, _ = make(24, 20, 5)
+    with mr.Plan(seq) as plan:
+        plan.set_slice_profile(8, 6, 0.2, 4.0, 2.0)
+        d = plan.forward(a, mask=mask)
+        outs = []
+        for x in (a, spoil(a, mask, value, slice(0, 2))):
+            x = x.clone()
+            x[:2, mask != 0] += 0.1
+            rep = plan.gn_solve(d, x, mask=mask, outer_iters=2, inner_iters=4)
+            outs.append((x[:, mask != 0], rep["f"], rep["f_final"]))
+    assert np.isfinite(outs[0][2])
+    assert torch.equal(outs[0][0], outs[1][0]) and outs[0][1:] == outs[1][1:]
