@@ -94,6 +94,10 @@ lr_project_kernel(const float* __restrict__ alpha, const float* __restrict__ b1,
     t2 = expf(alpha[nv + j]);
     if (B1MAP) bj = b1[j];
   }
+  // a voxel outside the mask stands for zeros whatever its parameters are (NaN too)
+  t1 = on ? t1 : 1000.f;
+  t2 = on ? t2 : 100.f;
+  if (B1MAP) bj = on ? bj : 1.f;
   const float x1 = expm1f(-tr / t1), x2 = expm1f(-tr / t2), x2e = expm1f(-te / t2);
   const float d1 = tr / t1 * (1.f + x1), d2 = tr / t2 * (1.f + x2);
   float my = 0.f, mz = m0z, ay = 0.f, az = 0.f, by = 0.f, bz = 0.f;

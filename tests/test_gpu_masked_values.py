@@ -76,3 +76,23 @@ def test_slice_profile_solve(value):
             outs.append((x[:, mask != 0], rep["f"], rep["f_final"]))
     assert np.isfinite(outs[0][2])
     assert torch.equal(outs[0][0], outs[1][0]) and outs[0][1:] == outs[1][1:]
+
+
+# 64 x 40: columns of 32 N rows; 33 x 20: the DFTs as GEMMs
+@pytest.mark.parametrize("value", BAD)
+@pytest.mark.parametrize("nx,ny,rank", [(40, 64, 32), (33, 20, 8)])
+@pytest.mark.parametrize("with_b1", [False, True])
+def test_lowrank_projection(with_b1, nx, ny, rank, value):
+    import paper_1904_13244_gb300 as mr
+    seq, a, mask, v, w = make(nx, ny, 4, extra=1)
+    U = torch.linalg.qr(torch.randn((seq.ntr, rank), generator=torch.Generator().manual_seed(3)))[0].cuda()
+    b1 = 0.9 + 0.2 * torch.rand(seq.nv, device="cuda") if with_b1 else None
+    bad, bad_b1 = spoil(a, mask, value, slice(0, 2)), spoil(b1[None], mask, value)[0] if with_b1 else None
+    with mr.Plan(seq) as plan:
+        plan.lowrank_set_basis(U.contiguous())
+        outs = []
+        for x, b in ((a, b1), (bad, bad_b1)):
+            plan.lowrank_linearize(x, b1=b, mask=mask)
+            outs.append([plan.lowrank_coefficients(), plan.jvp(v), plan.jhw(w), plan.jhjv(v), plan.cg_fixed(v, 3)])
+    assert all_equal(outs[1], outs[0])
+    assert not outs[1][0][..., mask == 0].any()
