@@ -383,8 +383,8 @@ __global__ void segment_sum_kernel(const float* __restrict__ zpart, const float*
   for (int s = 0; s < nseg; ++s)
 #pragma unroll
     for (int c = 0; c < 6; ++c) z[c] += zpart[((size_t)s * 6 + c) * nv + j];
-  const float m = (mask == nullptr || mask[j]) ? 1.f : 0.f;
-  const float rr = alpha[2 * (size_t)nv + j] * m, ri = alpha[3 * (size_t)nv + j] * m;
+  const bool on = mask == nullptr || mask[j] != 0;
+  const float m = on ? 1.f : 0.f, rr = on ? alpha[2 * (size_t)nv + j] : 0.f, ri = on ? alpha[3 * (size_t)nv + j] : 0.f;
   g[j] = (rr * z[3] - ri * z[2]) * m;
   g[nv + j] = (rr * z[5] - ri * z[4]) * m;
   g[2 * (size_t)nv + j] = z[1] * m;

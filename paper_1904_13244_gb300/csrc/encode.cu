@@ -28,17 +28,18 @@ __global__ void prep_forward_kernel(const float* __restrict__ alpha, const uint8
                                     int nv, float2* __restrict__ cf) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= nv) return;
-  const float m = (mask == nullptr || mask[j]) ? 1.f : 0.f;
-  cf[j] = make_float2(alpha[2 * nv + j] * m, alpha[3 * nv + j] * m);
+  // selected, not multiplied: rho outside the mask may be anything (NaN too)
+  const bool on = mask == nullptr || mask[j] != 0;
+  cf[j] = on ? make_float2(alpha[2 * nv + j], alpha[3 * nv + j]) : make_float2(0.f, 0.f);
 }
 
 __global__ void prep_linearize_kernel(const float* __restrict__ alpha, const uint8_t* __restrict__ mask,
                                       int nv, float2* __restrict__ rho, float* __restrict__ maskf) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= nv) return;
-  const float m = (mask == nullptr || mask[j]) ? 1.f : 0.f;
-  rho[j] = make_float2(alpha[2 * nv + j] * m, alpha[3 * nv + j] * m);
-  maskf[j] = m;
+  const bool on = mask == nullptr || mask[j] != 0;
+  rho[j] = on ? make_float2(alpha[2 * nv + j], alpha[3 * nv + j]) : make_float2(0.f, 0.f);
+  maskf[j] = on ? 1.f : 0.f;
 }
 
 __global__ void prep_rho_kernel(const float2* __restrict__ rho, int nv, float2* __restrict__ cf) {

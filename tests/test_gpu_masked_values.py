@@ -96,3 +96,28 @@ def test_lowrank_projection(with_b1, nx, ny, rank, value):
             outs.append([plan.lowrank_coefficients(), plan.jvp(v), plan.jhw(w), plan.jhjv(v), plan.cg_fixed(v, 3)])
     assert all_equal(outs[1], outs[0])
     assert not outs[1][0][..., mask == 0].any()
+
+
+@pytest.mark.parametrize("value", BAD)
+@pytest.mark.parametrize("model", ["slice", "b1", "estimated b1", "checkpointed b1", "recompute"])
+def test_proton_density(model, value):
+    import paper_1904_13244_gb300 as mr
+    seq, a, mask, v, w = make(29, 21, 4, extra=3, npar=5 if model == "estimated b1" else 4)
+    rows = slice(2, 4)
+    b1 = 0.9 + 0.2 * torch.rand(seq.nv, device="cuda") if model in ("b1", "checkpointed b1") else None
+    bad = spoil(a, mask, value, rows)
+    with mr.Plan(seq, estimate_b1=model == "estimated b1") as plan:
+        if model == "slice":
+            plan.set_slice_profile(16, 6, 0.2, 4.0, 2.0)
+        if model == "recompute":
+            plan.set_recompute(32)
+        outs = []
+        for x in (a, bad):
+            if model == "checkpointed b1":
+                outs.append([plan.forward_ckpt(x, b1=b1, mask=mask, interval=16), plan.jhw_ckpt(w)])
+            elif model == "recompute":
+                plan.linearize(x, mask=mask)
+                outs.append([plan.jvp(v), plan.jhw(w), plan.jhjv(v)])
+            else:
+                outs.append(exact_calls(plan, x, mask, v, w, b1=b1))
+    assert all_equal(outs[1], outs[0])
