@@ -101,17 +101,19 @@ __device__ __forceinline__ int rc_mod(int a, int n, unsigned magic) {
 // Linearisation: relaxation factors and the state before every seg-th TR, per voxel.
 //   rlx [8][nv]: x1a x2a d1a d2a x1b x2b d1b d2b;  ckpt [nseg][6][nv]
 __global__ void __launch_bounds__(128)
-rc_ckpt_kernel(const float* __restrict__ alpha, const float* __restrict__ b1, const float2* __restrict__ cs,
-               const float* __restrict__ phi, int nv, int ntr, int seg, int nseg, float te, float tb, float m0z,
-               float* __restrict__ rlx, float* __restrict__ ckpt) {
+rc_ckpt_kernel(const float* __restrict__ alpha, const float* __restrict__ b1, const float* __restrict__ maskf,
+               const float2* __restrict__ cs, const float* __restrict__ phi, int nv, int ntr, int seg, int nseg,
+               float te, float tb, float m0z, float* __restrict__ rlx, float* __restrict__ ckpt) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= nv) return;
-  const float t1 = expf(alpha[j]), t2 = expf(alpha[nv + j]);
+  // a voxel outside the mask stands for zeros whatever its parameters are (NaN too)
+  const bool on = maskf[j] != 0.f;
+  const float t1 = on ? expf(alpha[j]) : 1000.f, t2 = on ? expf(alpha[nv + j]) : 100.f;
   const RcRelax r = rc_relax(t1, t2, te, tb);
   const float rv[8] = {r.x1a, r.x2a, r.d1a, r.d2a, r.x1b, r.x2b, r.d1b, r.d2b};
 #pragma unroll
   for (int k = 0; k < 8; ++k) rlx[(size_t)k * nv + j] = rv[k];
-  const float bj = b1 != nullptr ? b1[j] : 1.f;
+  const float bj = b1 != nullptr && on ? b1[j] : 1.f;
   RcState s{0.f, m0z, 0.f, 0.f, 0.f, 0.f};
   for (int sg = 0; sg < nseg; ++sg) {
     float* c = ckpt + (size_t)sg * 6 * nv + j;
@@ -213,7 +215,7 @@ rc_product_kernel(const float* __restrict__ rlx, const float* __restrict__ ckpt,
              rlx[4 * (size_t)nv + j], rlx[5 * (size_t)nv + j], rlx[6 * (size_t)nv + j], rlx[7 * (size_t)nv + j]};
       const float* c = ckpt + (size_t)sg * 6 * nv + j;
       x.s = {c[0], c[(size_t)nv], c[2 * (size_t)nv], c[3 * (size_t)nv], c[4 * (size_t)nv], c[5 * (size_t)nv]};
-      if (b1 != nullptr) x.bj = b1[j];
+      if (b1 != nullptr && x.m != 0.f) x.bj = b1[j];  // as the linearisation took it
       if (MODE != RC_JHW) {
         x.v0 = v[j];
         x.v1 = v[(size_t)nv + j];
@@ -338,7 +340,7 @@ bool recompute_supported(const Plan& p) { return p.ny <= kMaxRows && p.npar == 4
 
 cudaError_t launch_rc_linearize(const Plan& p, const float* alpha, const float* b1, cudaStream_t st) {
   if (p.nv == 0) return cudaSuccess;
-  rc_ckpt_kernel<<<(p.nv + 127) / 128, 128, 0, st>>>(alpha, b1, p.cs, p.phi, p.nv, p.ntr, p.rc_seg, p.rc_nseg,
+  rc_ckpt_kernel<<<(p.nv + 127) / 128, 128, 0, st>>>(alpha, b1, p.maskf, p.cs, p.phi, p.nv, p.ntr, p.rc_seg, p.rc_nseg,
                                                      (float)p.te_ms, (float)(p.tr_ms - p.te_ms),
                                                      p.inversion ? -1.f : 1.f, p.rc_rlx, p.rc_ckpt);
   return cudaGetLastError();

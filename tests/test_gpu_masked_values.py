@@ -121,3 +121,19 @@ def test_proton_density(model, value):
             else:
                 outs.append(exact_calls(plan, x, mask, v, w, b1=b1))
     assert all_equal(outs[1], outs[0])
+
+
+@pytest.mark.parametrize("value", BAD)
+@pytest.mark.parametrize("with_b1", [False, True])
+def test_recompute_form(with_b1, value):
+    import paper_1904_13244_gb300 as mr
+    seq, a, mask, v, w = make(29, 21, 4, extra=3)
+    b1 = 0.9 + 0.2 * torch.rand(seq.nv, device="cuda") if with_b1 else None
+    bad, bad_b1 = spoil(a, mask, value), spoil(b1[None], mask, value)[0] if with_b1 else None
+    outs = []
+    with mr.Plan(seq) as plan:
+        plan.set_recompute(32)
+        for x, b in ((a, b1), (bad, bad_b1)):
+            plan.linearize(x, b1=b, mask=mask)
+            outs.append([plan.jvp(v), plan.jhw(w), plan.jhjv(v)])
+    assert all_equal(outs[1], outs[0])
