@@ -550,18 +550,26 @@ rx_product_kernel(const __grid_constant__ RxArgs P) {
   cl.sync();
   const int E = 4 * rows * kTX;
   const int ea = (int)((int64_t)E * sg / P.nseg), ee = (int)((int64_t)E * (sg + 1) / P.nseg);
+  // <v, g> and <v, v>: float32 over four elements at most, then float64
+  double a = 0.0, b = 0.0;
   float sd = 0.f, sv = 0.f;
+  int held = 0;
   for (int e = ea + tid; e < ee; e += nthr) {
-    float a = 0.f;
-    for (int q = 0; q < P.nseg; ++q) a += cl.map_shared_rank(gbuf, q)[e];
+    float t = 0.f;
+    for (int q = 0; q < P.nseg; ++q) t += cl.map_shared_rank(gbuf, q)[e];
     const int i = e / (rows * kTX), r = e / kTX - i * rows, col = tile * kTX + e % kTX;
     if (r < ny && col < nx) {
       const size_t j = (size_t)i * nv + (size_t)r * nx + col;
-      P.g[j] = a;
+      P.g[j] = t;
       if (MODE == RX_JHJV && P.vdot != nullptr) {
         const float vk = P.v[j];
-        sd = fmaf(vk, a, sd);
+        sd = fmaf(vk, t, sd);
         sv = fmaf(vk, vk, sv);
+        if ((++held & 3) == 0) {
+          a += (double)sd;
+          b += (double)sv;
+          sd = sv = 0.f;
+        }
       }
     }
   }
@@ -570,7 +578,8 @@ rx_product_kernel(const __grid_constant__ RxArgs P) {
   // <v, g> and <v, v>: this block's parts, then the last block adds all of them in order
   __shared__ double ws[2][kMaxWarps];
   __shared__ int s_last;
-  double a = red::warp_sum((double)sd), b = red::warp_sum((double)sv);
+  a = red::warp_sum(a + (double)sd);
+  b = red::warp_sum(b + (double)sv);
   if (lane == 0) {
     ws[0][warp] = a;
     ws[1][warp] = b;
