@@ -261,7 +261,8 @@ rx_product_kernel(const __grid_constant__ RxArgs P) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const bool o = on[k] && r0[k] + h < ny;
-      const int j = o ? (r0[k] + h) * nx + ix : 0;
+      // a row past the image reads row 0 of its own column: a NaN in v stays in its column
+      const int j = o ? (r0[k] + h) * nx + ix : min(ix, nx - 1);
       float2 rh = make_float2(0.f, 0.f);
       if (MODE != RX_JHW) rh = o ? P.rho[j] : rh;
       const float e = o ? P.fac[4 * nvp + ci[k] + h] : 0.f;
