@@ -775,6 +775,8 @@ int mrstat_gn_solve(mrstat_plan* plan_, const float* d, float* alpha, const floa
   if (e != cudaSuccess) return cuda_fail(e, "Gauss-Newton work space");
 
   Solver S{p, st, (int64_t)p->npar * p->nv, 2 * (int64_t)p->ntr * p->nkx, p->gn_sc, p->gn_si};
+  // the plan's linearisation is overwritten from here on; a solve that fails leaves none
+  p->linearized = false;
   if (p->lr) p->lr->active = false;
   bool coef_stale = true;  // low-rank coefficients of the current point
   const int nv = p->nv;

@@ -2166,6 +2166,7 @@ int lowrank_setup(Plan* p, const float* U_dev, int R, cudaStream_t st) {
     if (s != MRSTAT_OK) return s;
   }
   if (p->lr) {
+    if (p->lr->active) p->linearized = false;  // the linearisation goes with its basis
     lowrank_free(p->lr);
     p->lr = nullptr;
   }

@@ -1,0 +1,55 @@
+"""A plan whose linearisation is gone says so: a product then is an error, not a launch on
+buffers that were never filled.
+"""
+import numpy as np
+import pytest
+
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def setup():
+    import paper_1904_13244_gb300 as mr
+    seq = synth.make_sequence(12, 10, 4, 7.6, 3.8, seed=1)
+    rng = np.random.default_rng(1)
+    alpha = np.stack([rng.uniform(np.log(300), np.log(3000), seq.nv), rng.uniform(np.log(30), np.log(300), seq.nv),
+                      rng.uniform(0.5, 1, seq.nv), rng.uniform(-1, 1, seq.nv)])
+    U = torch.linalg.qr(torch.randn((seq.ntr, 8), generator=torch.Generator().manual_seed(3)))[0].contiguous().cuda()
+    dev = lambda a, t=torch.float32: torch.tensor(a, dtype=t, device="cuda")  # noqa: E731
+    return (mr, mr.Plan(seq), dev(alpha), U, dev(synth.random_params(seq.nv, 1)),
+            dev(synth.random_kspace(seq.ntr, seq.nkx, 2), torch.complex64))
+
+
+def refused(mr, plan, v, w):
+    for call in (lambda: plan.jvp(v), lambda: plan.jhw(w), lambda: plan.jhjv(v), lambda: plan.cg_fixed(v, 2),
+                 lambda: plan.timecourses(0)):
+        with pytest.raises(mr.MrstatError, match="(?i)lineari"):
+            call()
+
+
+def test_another_basis_drops_the_lowrank_linearisation():
+    mr, plan, a, U, v, w = setup()
+    with plan:
+        plan.lowrank_set_basis(U)
+        plan.lowrank_linearize(a)
+        plan.jvp(v)
+        plan.lowrank_set_basis(U)
+        refused(mr, plan, v, w)
+        plan.linearize(a)  # an exact linearisation stays when the basis changes
+        ref = plan.jhjv(v)
+        plan.lowrank_set_basis(U)
+        assert torch.equal(plan.jhjv(v), ref)
+
+
+def test_failed_solve_leaves_no_linearisation():
+    mr, plan, a, U, v, w = setup()
+    with plan:
+        plan.linearize(a)
+        ref = plan.jhjv(v)
+        with pytest.raises(mr.MrstatError, match="finite"):
+            plan.gn_solve(torch.full_like(w, float("nan")), a.clone(), outer_iters=1, inner_iters=2)
+        refused(mr, plan, v, w)
+        plan.linearize(a)
+        assert torch.equal(plan.jhjv(v), ref)
