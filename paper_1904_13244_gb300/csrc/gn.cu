@@ -517,7 +517,6 @@ void swap_ptr(T*& a, T*& b) {
 
 cudaError_t ensure_workspace(Plan* p) {
   if (p->gn_ready) return cudaSuccess;
-  if (ensure_timecourses(p) != cudaSuccess) return cudaErrorMemoryAllocation;
   const size_t nv = p->nv, nk = (size_t)p->ntr * p->nkx;
   cudaError_t e = cudaSuccess;
   auto chk = [&](cudaError_t r) {
@@ -618,14 +617,14 @@ struct Solver {
   }
 
   // The exact least-squares rho at a uniform point, nkx = nx and ny <= ntr (the k-space work
-  // arrays hold ny rows); m_n of its one time course in D (voxel stride nvd); solution rows
-  // 2..3 of gn_z
-  int ls_rho(const float* d, int nvd) {
+  // arrays hold ny rows); m_n of its one time course from the time courses D with voxel stride
+  // nvd; solution rows 2..3 of gn_z
+  int ls_rho(const float* d, const float4* D, int nvd) {
     const int nx = p->nx, ny = p->ny, nkx = p->nkx;
     cudaError_t e = cudaMemsetAsync(p->gn_z, 0, (size_t)p->npar * p->nv * sizeof(float), st);
     if (e == cudaSuccess)
       e = vec([&] {
-        rho_ls_kspace_kernel<<<ny, 256, 0, st>>>(reinterpret_cast<const float*>(p->D), nvd,
+        rho_ls_kspace_kernel<<<ny, 256, 0, st>>>(reinterpret_cast<const float*>(D), nvd,
                                                  reinterpret_cast<const float2*>(d), nkx, p->ky_ptr, p->ky_tr,
                                                  p->gn_jv);
       });
@@ -798,19 +797,20 @@ int mrstat_gn_solve(mrstat_plan* plan_, const float* d, float* alpha, const floa
     if (e != cudaSuccess) return cuda_fail(e, "rho init fill");
     if (o->rho_init_exact && rx_applies(p, b1)) {
       // one voxel's time course serves all of them
+      if (p->gn_course == nullptr) e = dalloc(p, &p->gn_course, (size_t)p->nch * p->nq);
+      if (e != cudaSuccess) return cuda_fail(e, "rho init time course");
       e = S.vec([&] {
         fill_rows_kernel<<<1, 32, 0, st>>>(p->gn_trial, 1, p->npar, (float)std::log(o->t1_init_ms),
                                            (float)std::log(o->t2_init_ms));
       });
       if (e == cudaSuccess) {
         Span sp(p, MRSTAT_K_BLOCH, st);
-        p->d_valid = false;
-        e = launch_bloch_n(*p, p->gn_trial, nullptr, p->D, 1, st);
+        e = launch_bloch_n(*p, p->gn_trial, nullptr, p->gn_course, 1, st);
       }
-      status = e == cudaSuccess ? S.ls_rho(d, 1) : cuda_fail(e, "rho init time course");
+      status = e == cudaSuccess ? S.ls_rho(d, p->gn_course, 1) : cuda_fail(e, "rho init time course");
     } else {
       status = do_linearize(p, p->gn_alpha, b1, nullptr, false, p->rho, st);
-      if (status == MRSTAT_OK) status = o->rho_init_exact ? S.ls_rho(d, p->nv) : S.cgls_rho(d, o->rho_init_iters);
+      if (status == MRSTAT_OK) status = o->rho_init_exact ? S.ls_rho(d, p->D, p->nv) : S.cgls_rho(d, o->rho_init_iters);
     }
     if (status != MRSTAT_OK) return status;
     const float* x = p->gn_z + 2 * (int64_t)nv;

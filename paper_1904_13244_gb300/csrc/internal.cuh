@@ -27,6 +27,7 @@ constexpr int kRedSlots = 16 * kRedBlocks;
 // A linearisation by recomputation (recur.cu): relaxation factors and the Bloch states before
 // every seg-th TR, column-major.
 struct RxLin {
+  float* mem = nullptr;  // its memory, NULL where it lies behind the time courses D
   float* fac = nullptr;  // [6][nx][nys]
   float* st = nullptr;   // [cap][ns][nx][nys], nseg of them in use
   int seg = 0, nseg = 0, cap = 0, ns = 6;
@@ -107,6 +108,7 @@ struct Plan {
   // recomputed linearisations of the exact model (hard pulses, no B1 map): the plan's, the
   // Gauss-Newton trial point's, the forward's (m alone) and the checkpointed forward's
   RxLin rx, rx2, rxf, rxc;
+  float4* gn_course = nullptr;      // [3][nq] one voxel's time courses (exact rho initialisation)
   int rx_seg = 0;                   // TRs per segment
   bool rx_active = false;           // the current exact linearisation is rx (else D)
   bool d_valid = false;             // D holds its time courses
@@ -239,7 +241,7 @@ int do_jhjv(Plan* p, const float* v, float* out, cudaStream_t st, double* vdot =
 int do_xdft(Plan* p, const float2* A, float2* out, const int* gate, cudaStream_t st);
 int do_xdft_adj(Plan* p, const float2* w, float2* out, const int* gate, cudaStream_t st);
 
-cudaError_t ensure_timecourses(Plan* p);   // allocates D on first use
+cudaError_t ensure_timecourses(Plan* p);   // allocates D on first use (forms that store or ask for it)
 int build_split_tables(Plan* p);           // split-BF16 readout DFT operands (plan.cu)
 // low-rank form (lowrank.cu)
 int lowrank_setup(Plan* p, const float* U_dev, int R, cudaStream_t st);

@@ -46,8 +46,8 @@ void free_plan(Plan* p) {
                   p->gn_dir, p->gn_q, p->gn_alpha, p->gn_trial, p->gn_s, p->gn_r, p->gn_st,
                   p->gn_rt, p->gn_jv, p->gn_mask, p->gn_sc, p->gn_si, p->bf_ft_hi, p->bf_ft_lo,
                   p->bf_fh_hi, p->bf_fh_lo, p->bf_a_hi, p->bf_a_lo, p->bf_w_hi, p->bf_w_lo, p->dev_err, p->ckpt, p->zpart,
-                  p->rc_rlx, p->rc_ckpt, p->rc_gpart, p->rc_b1, p->csp, p->rx.fac, p->rx.st, p->rx2.fac, p->rx2.st,
-                  p->rxf.fac, p->rxf.st, p->rxc.fac, p->rxc.st, p->rx_ticket, p->rx_etab, p->rxc_rho, p->rxc_maskf};
+                  p->rc_rlx, p->rc_ckpt, p->rc_gpart, p->rc_b1, p->csp, p->rx.mem, p->rx2.mem, p->rxf.mem,
+                  p->rxc.mem, p->gn_course, p->rx_ticket, p->rx_etab, p->rxc_rho, p->rxc_maskf};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   for (cudaEvent_t e : p->event_pool) cudaEventDestroy(e);
@@ -89,25 +89,59 @@ bool rx_applies(const Plan* p, const float* b1) {
 
 namespace {
 
-// Allocates L (once per segment length) with ns floats per state.
+size_t rx_fac_floats(const Plan& p) { return (6 * (size_t)p.nx * rx_nys(p) + 63) / 64 * 64; }
+
+size_t rx_floats(const Plan& p, int ns, int nseg) {
+  return rx_fac_floats(p) + (size_t)nseg * ns * p.nx * rx_nys(p);
+}
+
+void rx_place(const Plan& p, RxLin* L, float* mem, int ns, int nseg) {
+  L->fac = mem;
+  L->st = mem + rx_fac_floats(p);
+  L->ns = ns;
+  L->cap = L->nseg = nseg;
+}
+
+// Allocates L with ns floats per state, again where it needs more segments than it has.
 cudaError_t ensure_rx(Plan* p, RxLin* L, int ns, int seg) {
-  const size_t nvp = (size_t)p->nx * rx_nys(*p);
   const int nseg = (p->ntr + seg - 1) / seg;
-  cudaError_t e = cudaSuccess;
-  if (L->fac == nullptr) e = dalloc(p, &L->fac, 6 * nvp);
-  if (e == cudaSuccess && L->st != nullptr && L->cap < nseg) {
-    e = cudaDeviceSynchronize();
-    cudaFree(L->st);
-    p->bytes -= (int64_t)((size_t)L->cap * L->ns * nvp * sizeof(float));
-    L->st = nullptr;
+  if (L->fac != nullptr && L->cap >= nseg) {
+    L->nseg = nseg;
+    return cudaSuccess;
   }
-  if (e == cudaSuccess && L->st == nullptr) {
-    e = dalloc(p, &L->st, (size_t)nseg * ns * nvp);
-    L->ns = ns;
-    L->cap = nseg;
+  if (L->mem != nullptr) {
+    const cudaError_t e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) return e;
+    cudaFree(L->mem);
+    p->bytes -= (int64_t)(rx_floats(*p, L->ns, L->cap) * sizeof(float));
+    *L = RxLin();
   }
-  L->nseg = nseg;
+  const cudaError_t e = dalloc(p, &L->mem, rx_floats(*p, ns, nseg));
+  if (e == cudaSuccess) rx_place(*p, L, L->mem, ns, nseg);
   return e;
+}
+
+// The memory of a plan's first recomputed linearisation: the time courses D, which
+// mrstat_timecourses fills, and behind them what the products read, in one allocation (a
+// cudaMalloc takes 31-37 us from 1 to 100 MB, 90 us at 674 MB: three of them were a third of
+// a small plan's first pass).  No product needs D, so where it does not fit it is left out.
+cudaError_t reserve_linearization(Plan* p) {
+  if (p->rx.fac == nullptr && p->D == nullptr) {
+    const int nseg = (p->ntr + p->rx_seg - 1) / p->rx_seg;
+    const size_t d = (size_t)p->nch * p->nq * p->nv;
+    const size_t behind = (d + 15) / 16 * 16;  // 256-byte aligned
+    const cudaError_t e = dalloc(p, &p->D, behind + (rx_floats(*p, 6, nseg) + 3) / 4);
+    if (e == cudaSuccess) {
+      p->d_bytes = (int64_t)(d * sizeof(float4));
+      rx_place(*p, &p->rx, reinterpret_cast<float*>(p->D + behind), 6, nseg);
+    } else if (e == cudaErrorMemoryAllocation) {
+      p->D = nullptr;
+      cudaGetLastError();
+    } else {
+      return e;
+    }
+  }
+  return ensure_rx(p, &p->rx, 6, p->rx_seg);
 }
 
 }  // namespace
@@ -312,17 +346,17 @@ int do_linearize(Plan* p, const float* alpha, const float* b1, const uint8_t* ma
   if (!trial) p->d_valid = false;
   if (p->rx_active) {
     RxLin* L = trial ? &p->rx2 : &p->rx;
-    e = ensure_rx(p, L, 6, p->rx_seg);
+    e = ensure_rx(p, L, 6, p->rx_seg);  // mrstat_linearize has reserved the plan's own
     if (e != cudaSuccess) return cuda_fail(e, "linearisation allocation");
     Span sp(p, MRSTAT_K_BLOCH, st);
     L->seg = p->rx_seg;
     e = launch_rx_states(*p, *L, alpha, mask, rho, p->maskf, st);
     return e == cudaSuccess ? MRSTAT_OK : cuda_fail(e, "linearisation launch");
   }
-  if (trial && p->D2 == nullptr) {
-    e = dalloc(p, &p->D2, (size_t)p->nch * p->nq * p->nv);
-    if (e != cudaSuccess) return cuda_fail(e, "time-course allocation");
-  }
+  e = cudaSuccess;
+  if (!trial) e = ensure_timecourses(p);
+  else if (p->D2 == nullptr) e = dalloc(p, &p->D2, (size_t)p->nch * p->nq * p->nv);
+  if (e != cudaSuccess) return cuda_fail(e, "time-course allocation");
   {
     Span sp(p, MRSTAT_K_VECTOR, st);
     e = launch_prep_linearize(*p, alpha, mask, rho, st);
@@ -696,8 +730,10 @@ int mrstat_linearize(mrstat_plan* plan, const float* alpha, const float* b1, con
     plan->linearized = true;
     return MRSTAT_OK;
   }
-  cudaError_t ea = ensure_timecourses(plan);
-  if (ea != cudaSuccess) return cuda_fail(ea, "time-course allocation");
+  if (rx_applies(plan, b1)) {
+    const cudaError_t e = reserve_linearization(plan);
+    if (e != cudaSuccess) return cuda_fail(e, "linearisation allocation");
+  }
   const int status = do_linearize(plan, alpha, b1, mask, false, plan->rho, st);
   if (status != MRSTAT_OK) return status;
   plan->linearized = true;
@@ -780,12 +816,15 @@ int mrstat_timecourses(mrstat_plan* plan, int32_t channel, float* out, void* str
   if (channel < 0 || channel >= plan->nch)
     return fail(MRSTAT_ERR_INVALID_ARG, "channel %d not in [0, %d)", channel, plan->nch);
   if (plan->rc_seg > 0) return fail(MRSTAT_ERR_UNSUPPORTED, "the recompute form keeps no time courses");
-  if (!plan->linearized || plan->D == nullptr || (plan->lr && plan->lr->active))
+  if (!plan->linearized || (plan->lr && plan->lr->active))
     return fail(MRSTAT_ERR_NOT_LINEARIZED, "timecourses need an exact mrstat_linearize");
   DeviceGuard g(plan->device);
   if (plan->rx_active && !plan->d_valid) {  // all channels, from the kept states
+    // D was reserved by mrstat_linearize; a solve or a plan short of memory has none yet
+    cudaError_t e = ensure_timecourses(plan);
+    if (e != cudaSuccess) return cuda_fail(e, "time-course allocation");
     Span sp(plan, MRSTAT_K_BLOCH, as_stream(stream));
-    const cudaError_t e = launch_rx_expand(*plan, plan->rx, plan->D, as_stream(stream));
+    e = launch_rx_expand(*plan, plan->rx, plan->D, as_stream(stream));
     if (e != cudaSuccess) return cuda_fail(e, "timecourse launch");
     plan->d_valid = true;
   }
