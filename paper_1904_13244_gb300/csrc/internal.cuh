@@ -48,7 +48,6 @@ struct Plan {
   // per-TR tables (device)
   float2* cs = nullptr;     // [ntr_pad] (cos phi_n, sin phi_n), phi_n the signed flip
   float* phi = nullptr;     // [ntr_pad] signed flip (radians)
-  float4* csp = nullptr;    // [ntr_pad][2] (c, c, s, s), (-s, -s, 0, 0) of the signed flip
   // slice profile (mrstat_set_slice_profile): 0 isochromats = hard pulses
   int slice_iso = 0, slice_sub = 0;
   float* slice_rot = nullptr;    // [ntr_pad][pairs][10][2] composed pulses of each TR and isochromat pair (slice.cu)
@@ -112,8 +111,10 @@ struct Plan {
   int rx_seg = 0;                   // TRs per segment
   bool rx_active = false;           // the current exact linearisation is rx (else D)
   bool d_valid = false;             // D holds its time courses
+  float4* rx_tab = nullptr;         // memory of the next three (recur.cu)
+  float4* csp = nullptr;            // [ntr_pad][2] (c, c, s, s), (-s, -s, 0, 0) of the signed flip
+  float4* rx_etab = nullptr;        // [ny][row pairs] phases
   unsigned* rx_ticket = nullptr;    // zero between launches
-  float4* rx_etab = nullptr;        // [ny][row pairs] phases (recur.cu)
   float2* rxc_rho = nullptr;        // [nv] masked rho and mask of the checkpointed forward
   float* rxc_maskf = nullptr;
   bool rxc_active = false;          // the checkpointed forward kept rxc (else ckpt)
@@ -320,7 +321,7 @@ cudaError_t launch_timecourse(const Plan& p, int channel, float* out, cudaStream
 inline int rx_nys(const Plan& p) { return (p.ny + 1) / 2 * 2; }
 bool rx_supported(const Plan& p);
 int rx_segment(const Plan& p, int sms);
-std::vector<float4> rx_phase_table(const Plan& p, const std::vector<float2>& roots);
+cudaError_t rx_tables(Plan* p);
 cudaError_t launch_rx_states(const Plan& p, const RxLin& L, const float* alpha, const uint8_t* mask, float2* rho,
                              float* maskf, cudaStream_t st);
 cudaError_t launch_rx_signal(const Plan& p, const RxLin& L, const float2* rho, cudaStream_t st);

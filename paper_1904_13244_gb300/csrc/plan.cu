@@ -46,8 +46,8 @@ void free_plan(Plan* p) {
                   p->gn_dir, p->gn_q, p->gn_alpha, p->gn_trial, p->gn_s, p->gn_r, p->gn_st,
                   p->gn_rt, p->gn_jv, p->gn_mask, p->gn_sc, p->gn_si, p->bf_ft_hi, p->bf_ft_lo,
                   p->bf_fh_hi, p->bf_fh_lo, p->bf_a_hi, p->bf_a_lo, p->bf_w_hi, p->bf_w_lo, p->dev_err, p->ckpt, p->zpart,
-                  p->rc_rlx, p->rc_ckpt, p->rc_gpart, p->rc_b1, p->csp, p->rx.mem, p->rx2.mem, p->rxf.mem,
-                  p->rxc.mem, p->gn_course, p->rx_ticket, p->rx_etab, p->rxc_rho, p->rxc_maskf};
+                  p->rc_rlx, p->rc_ckpt, p->rc_gpart, p->rc_b1, p->rx.mem, p->rx2.mem, p->rxf.mem,
+                  p->rxc.mem, p->gn_course, p->rx_tab, p->rxc_rho, p->rxc_maskf};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   for (cudaEvent_t e : p->event_pool) cudaEventDestroy(e);
@@ -570,7 +570,6 @@ int mrstat_plan_create(const mrstat_seq* seq, int32_t form, mrstat_plan** out) {
 
   // host tables (float64, rounded once)
   std::vector<float2> cs(p->ntr_pad);
-  std::vector<float4> csp(2 * (size_t)p->ntr_pad);
   std::vector<float> phi(p->ntr_pad, 0.f);
   std::vector<int> kyi(p->ntr_pad, 0);
   for (int n = 0; n < p->ntr_pad; ++n) {
@@ -582,8 +581,6 @@ int mrstat_plan_create(const mrstat_seq* seq, int32_t form, mrstat_plan** out) {
     }
     phi[n] = (float)ph;
     cs[n] = make_float2((float)std::cos(ph), (float)std::sin(ph));
-    csp[2 * n] = make_float4(cs[n].x, cs[n].x, cs[n].y, cs[n].y);
-    csp[2 * n + 1] = make_float4(-cs[n].y, -cs[n].y, 0.f, 0.f);
   }
   std::vector<int> ky_ptr(p->ny + 1, 0), ky_tr(std::max(p->ntr, 1), 0);
   for (int n = 0; n < p->ntr; ++n) ky_ptr[kyi[n] + 1]++;
@@ -601,22 +598,12 @@ int mrstat_plan_create(const mrstat_seq* seq, int32_t form, mrstat_plan** out) {
       unit_root(kx * ix, p->nx, &fh[(size_t)k * p->nx + ix], true);
     }
 
-  std::vector<float4> rx_etab;
   const size_t nv = p->nv, nq = p->nq;
   cudaError_t e = cudaSuccess;
   auto chk = [&](cudaError_t r) {
     if (e == cudaSuccess) e = r;
   };
   chk(dalloc(p, &p->cs, p->ntr_pad));
-  chk(dalloc(p, &p->csp, csp.size()));
-  if (rx_supported(*p)) {
-    int sms = 0;
-    chk(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device));
-    p->rx_seg = rx_segment(*p, sms);
-    chk(dalloc(p, &p->rx_ticket, 1));
-    rx_etab = rx_phase_table(*p, roots);
-    chk(dalloc(p, &p->rx_etab, rx_etab.size()));
-  }
   chk(dalloc(p, &p->phi, p->ntr_pad));
   chk(dalloc(p, &p->kyi, p->ntr_pad));
   chk(dalloc(p, &p->roots, p->ny));
@@ -646,13 +633,15 @@ int mrstat_plan_create(const mrstat_seq* seq, int32_t form, mrstat_plan** out) {
     return st;
   }
   chk(cudaMemcpy(p->cs, cs.data(), cs.size() * sizeof(float2), cudaMemcpyHostToDevice));
-  chk(cudaMemcpy(p->csp, csp.data(), csp.size() * sizeof(float4), cudaMemcpyHostToDevice));
-  if (p->rx_etab)
-    chk(cudaMemcpy(p->rx_etab, rx_etab.data(), rx_etab.size() * sizeof(float4), cudaMemcpyHostToDevice));
-  if (p->rx_ticket) chk(cudaMemset(p->rx_ticket, 0, sizeof(unsigned)));
   chk(cudaMemcpy(p->phi, phi.data(), phi.size() * sizeof(float), cudaMemcpyHostToDevice));
   chk(cudaMemcpy(p->kyi, kyi.data(), kyi.size() * sizeof(int), cudaMemcpyHostToDevice));
   chk(cudaMemcpy(p->roots, roots.data(), roots.size() * sizeof(float2), cudaMemcpyHostToDevice));
+  if (rx_supported(*p)) {
+    int sms = 0;
+    chk(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device));
+    p->rx_seg = rx_segment(*p, sms);
+    chk(rx_tables(p));
+  }
   chk(cudaMemcpy(p->ky_ptr, ky_ptr.data(), ky_ptr.size() * sizeof(int), cudaMemcpyHostToDevice));
   chk(cudaMemcpy(p->ky_tr, ky_tr.data(), ky_tr.size() * sizeof(int), cudaMemcpyHostToDevice));
   chk(cudaMemcpy(p->ft, ft.data(), ft.size() * sizeof(float2), cudaMemcpyHostToDevice));
