@@ -42,6 +42,7 @@ struct Plan {
   int npar = 4;      // unknowns per voxel (5 with B1 estimated)
   int nch = 3;       // cached time-course channels (4 with B1 estimated)
   int device = 0;
+  int sms = 1;       // streaming multiprocessors of the device
   double tr_ms = 0, te_ms = 0;
   int inversion = 0, alternate = 0;
 

@@ -636,10 +636,9 @@ int mrstat_plan_create(const mrstat_seq* seq, int32_t form, mrstat_plan** out) {
   chk(cudaMemcpy(p->phi, phi.data(), phi.size() * sizeof(float), cudaMemcpyHostToDevice));
   chk(cudaMemcpy(p->kyi, kyi.data(), kyi.size() * sizeof(int), cudaMemcpyHostToDevice));
   chk(cudaMemcpy(p->roots, roots.data(), roots.size() * sizeof(float2), cudaMemcpyHostToDevice));
+  chk(cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device));
   if (rx_supported(*p)) {
-    int sms = 0;
-    chk(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device));
-    p->rx_seg = rx_segment(*p, sms);
+    p->rx_seg = rx_segment(*p, p->sms);
     chk(rx_tables(p));
   }
   chk(cudaMemcpy(p->ky_ptr, ky_ptr.data(), ky_ptr.size() * sizeof(int), cudaMemcpyHostToDevice));

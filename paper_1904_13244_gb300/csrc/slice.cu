@@ -219,7 +219,7 @@ template <int L>
 cudaError_t launch_slice(const Plan& p, const float* alpha, const uint8_t* mask, float4* D, int nch, cudaStream_t st) {
   if (nch > 1) return launch_slice_t<L, 3, 1>(p, alpha, mask, D, st);
   const int64_t warps = ((int64_t)p.nv * L + 31) / 32;
-  return warps >= 4 * 8 * 152 ? launch_slice_t<L, 1, 4>(p, alpha, mask, D, st)
+  return warps >= 4 * 8 * (int64_t)p.sms ? launch_slice_t<L, 1, 4>(p, alpha, mask, D, st)
                               : launch_slice_t<L, 1, 1>(p, alpha, mask, D, st);
 }
 
