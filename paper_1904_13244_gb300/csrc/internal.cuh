@@ -111,7 +111,6 @@ struct Plan {
   float4* gn_course = nullptr;      // [3][nq] one voxel's time courses (exact rho initialisation)
   int rx_seg = 0;                   // TRs per segment
   bool rx_active = false;           // the current exact linearisation is rx (else D)
-  bool d_valid = false;             // D holds its time courses
   float4* rx_tab = nullptr;         // memory of the next three (recur.cu)
   float4* csp = nullptr;            // [ntr_pad][2] (c, c, s, s), (-s, -s, 0, 0) of the signed flip
   float4* rx_etab = nullptr;        // [ny][row pairs] phases
@@ -243,7 +242,7 @@ int do_jhjv(Plan* p, const float* v, float* out, cudaStream_t st, double* vdot =
 int do_xdft(Plan* p, const float2* A, float2* out, const int* gate, cudaStream_t st);
 int do_xdft_adj(Plan* p, const float2* w, float2* out, const int* gate, cudaStream_t st);
 
-cudaError_t ensure_timecourses(Plan* p);   // allocates D on first use (forms that store or ask for it)
+cudaError_t ensure_timecourses(Plan* p);   // allocates D on first use
 int build_split_tables(Plan* p);           // split-BF16 readout DFT operands (plan.cu)
 // low-rank form (lowrank.cu)
 int lowrank_setup(Plan* p, const float* U_dev, int R, cudaStream_t st);
@@ -331,7 +330,7 @@ cudaError_t launch_rx_jhw(const Plan& p, const RxLin& L, const float2* rho, cons
                           float* g, cudaStream_t st);
 cudaError_t launch_rx_jhjv(const Plan& p, const RxLin& L, const float* v, float* g, double* vdot, double* vv,
                            cudaStream_t st);
-cudaError_t launch_rx_expand(const Plan& p, const RxLin& L, float4* D, cudaStream_t st);
+cudaError_t launch_rx_timecourse(const Plan& p, const RxLin& L, int channel, float* out, cudaStream_t st);
 // dft.cu
 cudaError_t launch_cgemm(const float2* A, const float2* B, float2* C, int M, int N, int K,
                          const int* gate, cudaStream_t st);

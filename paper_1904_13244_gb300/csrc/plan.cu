@@ -121,10 +121,11 @@ cudaError_t ensure_rx(Plan* p, RxLin* L, int ns, int seg) {
   return e;
 }
 
-// The memory of a plan's first recomputed linearisation: the time courses D, which
-// mrstat_timecourses fills, and behind them what the products read, in one allocation (a
-// cudaMalloc takes 31-37 us from 1 to 100 MB, 90 us at 674 MB: three of them were a third of
-// a small plan's first pass).  No product needs D, so where it does not fit it is left out.
+// The memory of a plan's first recomputed linearisation: what its products read, behind the
+// time courses D of a stored one, so that a later linearisation with a B1 map allocates
+// nothing (it may be captured).  One allocation: a cudaMalloc takes 31-37 us from 1 to 100 MB,
+// 90 us at 674 MB, and three of them were a third of a small plan's first pass.  The
+// recomputed form itself never reads D, so where D does not fit it is left out.
 cudaError_t reserve_linearization(Plan* p) {
   if (p->rx.fac == nullptr && p->D == nullptr) {
     const int nseg = (p->ntr + p->rx_seg - 1) / p->rx_seg;
@@ -295,10 +296,9 @@ int do_signal(Plan* p, bool trial, const float2* rho_masked, float2* s, cudaStre
 }
 
 void swap_linearisations(Plan* p) {
-  if (p->rx_active) std::swap(p->rx, p->rx2);  // D stays: it is only filled on demand
+  if (p->rx_active) std::swap(p->rx, p->rx2);
   else std::swap(p->D, p->D2);
   std::swap(p->rho, p->rho2);
-  p->d_valid = false;
 }
 
 int do_xdft(Plan* p, const float2* A, float2* out, const int* gate, cudaStream_t st) {
@@ -343,7 +343,6 @@ int do_linearize(Plan* p, const float* alpha, const float* b1, const uint8_t* ma
                  cudaStream_t st) {
   cudaError_t e;
   p->rx_active = rx_applies(p, b1);
-  if (!trial) p->d_valid = false;
   if (p->rx_active) {
     RxLin* L = trial ? &p->rx2 : &p->rx;
     e = ensure_rx(p, L, 6, p->rx_seg);  // mrstat_linearize has reserved the plan's own
@@ -371,7 +370,6 @@ int do_linearize(Plan* p, const float* alpha, const float* b1, const uint8_t* ma
                          : launch_bloch(*p, alpha, b1, mask, D, p->nch, st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "bloch launch");
-  if (!trial) p->d_valid = true;
   return MRSTAT_OK;
 }
 
@@ -807,14 +805,10 @@ int mrstat_timecourses(mrstat_plan* plan, int32_t channel, float* out, void* str
   if (!plan->linearized || (plan->lr && plan->lr->active))
     return fail(MRSTAT_ERR_NOT_LINEARIZED, "timecourses need an exact mrstat_linearize");
   DeviceGuard g(plan->device);
-  if (plan->rx_active && !plan->d_valid) {  // all channels, from the kept states
-    // D was reserved by mrstat_linearize; a solve or a plan short of memory has none yet
-    cudaError_t e = ensure_timecourses(plan);
-    if (e != cudaSuccess) return cuda_fail(e, "time-course allocation");
+  if (plan->rx_active) {  // from the kept states: nothing of an earlier call is reused
     Span sp(plan, MRSTAT_K_BLOCH, as_stream(stream));
-    e = launch_rx_expand(*plan, plan->rx, plan->D, as_stream(stream));
-    if (e != cudaSuccess) return cuda_fail(e, "timecourse launch");
-    plan->d_valid = true;
+    const cudaError_t e = launch_rx_timecourse(*plan, plan->rx, channel, out, as_stream(stream));
+    return e == cudaSuccess ? MRSTAT_OK : cuda_fail(e, "timecourse launch");
   }
   Span sp(plan, MRSTAT_K_VECTOR, as_stream(stream));
   cudaError_t e = launch_timecourse(*plan, channel, out, as_stream(stream));

@@ -617,49 +617,50 @@ rx_product_kernel(const __grid_constant__ RxArgs P) {
   }
 }
 
-// Time courses of one voxel and segment per thread from the kept states, as TR quads
-// D[c][n / 4][j] (mrstat_timecourses).
+// One time course channel (0 m_y, 1 and 2 its ln T1 and ln T2 tangents) of one voxel and
+// segment per thread, from the kept states into out[n][j] (mrstat_timecourses).
+template <int C>
 __global__ void __launch_bounds__(128)
-rx_expand_kernel(const float* __restrict__ fac, const float* __restrict__ st, const float* __restrict__ maskf,
-                 const float4* __restrict__ csp, int nx, int nys, int nv, int nq, int ntr, int seg,
-                 float4* __restrict__ D) {
+rx_timecourse_kernel(const float* __restrict__ fac, const float* __restrict__ st, const float* __restrict__ maskf,
+                     const float4* __restrict__ csp, int nx, int nys, int nv, int ntr, int seg, float* __restrict__ out) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x, sg = blockIdx.y;
   if (j >= nv) return;
-  const size_t nvp = (size_t)nx * nys, e = (size_t)(j % nx) * nys + j / nx, cstride = (size_t)nq * nv;
+  const size_t nvp = (size_t)nx * nys, e = (size_t)(j % nx) * nys + j / nx;
   const float x1 = fac[e], x2 = fac[nvp + e], d1 = fac[2 * nvp + e], d2 = fac[3 * nvp + e], ee = fac[4 * nvp + e],
               de = fac[5 * nvp + e];
   const float* s0 = st + (size_t)sg * 6 * nvp + e;
   float my = s0[0], mz = s0[nvp], ay = s0[2 * nvp], az = s0[3 * nvp], by = s0[4 * nvp], bz = s0[5 * nvp];
   const float m = maskf[j];
-  for (int n0 = sg * seg; n0 < min(ntr, (sg + 1) * seg); n0 += 4) {
-    float o[3][4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float4 cs = __ldg(csp + 2 * (n0 + k));  // the table is padded to whole quads
-      const float c = cs.x, s = cs.z;
-      float t = c * my + s * mz;
-      mz = c * mz - s * my;
-      my = t;
+  const int ne = min(ntr, (sg + 1) * seg);
+#pragma unroll 4
+  for (int n = sg * seg; n < ne; ++n) {
+    const float4 cs = __ldg(csp + 2 * n);
+    const float c = cs.x, s = cs.z;
+    float t = c * my + s * mz;
+    mz = c * mz - s * my;
+    my = t;
+    if (C == 1) {
       t = c * ay + s * az;
       az = c * az - s * ay;
       ay = t;
+    }
+    if (C == 2) {
       t = c * by + s * bz;
       bz = c * bz - s * by;
       by = t;
-      o[0][k] = m * ee * my;
-      o[1][k] = m * ee * ay;
-      o[2][k] = m * fmaf(ee, by, de * my);
-      const float zm1 = mz - 1.f;
+    }
+    __stcs(out + (size_t)n * nv + j, C == 0 ? m * ee * my : C == 1 ? m * ee * ay : m * fmaf(ee, by, de * my));
+    const float zm1 = mz - 1.f;
+    if (C == 1) {
       ay = fmaf(x2, ay, ay);
       az = fmaf(x1, az, fmaf(d1, zm1, az));
+    }
+    if (C == 2) {
       by = fmaf(x2, by, fmaf(d2, my, by));
       bz = fmaf(x1, bz, bz);
-      my = fmaf(x2, my, my);
-      mz = fmaf(x1, zm1, mz);
     }
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-      __stcs(D + c * cstride + (size_t)(n0 >> 2) * nv + j, make_float4(o[c][0], o[c][1], o[c][2], o[c][3]));
+    my = fmaf(x2, my, my);
+    mz = fmaf(x1, zm1, mz);
   }
 }
 
@@ -826,10 +827,11 @@ cudaError_t launch_rx_jhjv(const Plan& p, const RxLin& L, const float* v, float*
   return launch_product_t<3, RX_JHJV>(p, a, st);
 }
 
-cudaError_t launch_rx_expand(const Plan& p, const RxLin& L, float4* D, cudaStream_t st) {
+cudaError_t launch_rx_timecourse(const Plan& p, const RxLin& L, int channel, float* out, cudaStream_t st) {
   if (p.nv == 0) return cudaSuccess;
   const dim3 grid((p.nv + 127) / 128, L.nseg);
-  rx_expand_kernel<<<grid, 128, 0, st>>>(L.fac, L.st, p.maskf, p.csp, p.nx, rx_nys(p), p.nv, p.nq, p.ntr, L.seg, D);
+  auto kernel = channel == 0 ? rx_timecourse_kernel<0> : channel == 1 ? rx_timecourse_kernel<1> : rx_timecourse_kernel<2>;
+  kernel<<<grid, 128, 0, st>>>(L.fac, L.st, p.maskf, p.csp, p.nx, rx_nys(p), p.nv, p.ntr, L.seg, out);
   return cudaGetLastError();
 }
 

@@ -53,3 +53,33 @@ def test_failed_solve_leaves_no_linearisation():
         refused(mr, plan, v, w)
         plan.linearize(a)
         assert torch.equal(plan.jhjv(v), ref)
+
+
+def test_captured_calls_follow_the_linearisation():
+    """A captured product or time course reads the plan's linearisation when it is replayed, and a
+    captured linearisation serves the calls after its replay."""
+    mr, plan, a, U, v, w = setup()
+    b = a + 0.2
+    with plan:
+        def calls():
+            return [plan.timecourses(c) for c in range(3)] + [plan.jvp(v), plan.jhw(w), plan.jhjv(v)]
+
+        plan.linearize(b)
+        ref = calls()
+        x = a.clone()
+        plan.linearize(x)
+        old = calls()
+        torch.cuda.synchronize()
+        reads, lin = torch.cuda.CUDAGraph(), torch.cuda.CUDAGraph()
+        with torch.cuda.graph(reads):
+            out = calls()
+        with torch.cuda.graph(lin):
+            plan.linearize(x)
+        plan.linearize(b)
+        reads.replay()
+        assert all(torch.equal(p, q) for p, q in zip(out, ref))
+        lin.replay()
+        assert all(torch.equal(p, q) for p, q in zip(calls(), old))
+        x.copy_(b)
+        lin.replay()
+        assert all(torch.equal(p, q) for p, q in zip(calls(), ref))
