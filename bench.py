@@ -576,7 +576,7 @@ def differentiation(mr, torch, seq, ph, reps=10):
     """The differentiation form at the workload's size: s(alpha) as a torch.autograd.Function
     with the loss 1/2 ||s - d||^2, forward and backward timed with CUDA events (median of
     reps after a warm-up), with Bloch-state checkpoints every 64 TRs (the backward re-runs
-    the recursion segment by segment) and without (the forward caches the time courses);
+    the recursion segment by segment) and without (the plan's own linearisation and adjoint);
     device memory held by the plan after the forward, and torch's peak over the pass."""
     from paper_1904_13244_gb300.autograd import signal
     a0 = torch.tensor(alpha_of(ph), device="cuda")
@@ -614,7 +614,7 @@ def differentiation(mr, torch, seq, ph, reps=10):
 
 
 def plain_products(mr, torch, names=("ellipse64", "brain224"), reps=20):
-    """The plain FP32 form's single products per second (cached time courses): J.v,
+    """The plain FP32 form's single products per second: J.v,
     Re(J^H w) and Re(J^H J) v on the 64 x 64 / 320-TR ellipse workload and on brain224, CUDA
     events around reps back-to-back calls after a warm-up; the linearisation (K1) timed on
     its own."""
@@ -816,14 +816,14 @@ def main():
     # the plain FP32 form on the same inputs, for the comparison the metric asks for
     plain = None
     if args.form not in ("plain", "recompute"):
-        # the plain FP32 form in both variants, the plan's own (key "stored": the recursion
-        # re-run in packed pairs; time courses are stored only where that does not apply) and
+        # the plain FP32 form in both variants, the plan's own (key "default": the recursion
+        # re-run in packed pairs, or stored time courses past 256 rows) and
         # mrstat_set_recompute's (states every `segment` TRs); the faster one is the plain form
         # the comparison uses
         pplan = mr.Plan(seq)
         nst = max(1, args.steps // 4)
         pms, pstats, _ = timed(pplan, make_step(pplan, "plain"), nst, all_kernels)
-        stored = {"value": world * iters / (pms / 1e3), "ms_per_step": pms,
+        default = {"value": world * iters / (pms / 1e3), "ms_per_step": pms,
                   "kernel_ms_per_step": {k: pstats[k]["ms"] / nst for k in all_kernels}}
         pplan.set_recompute(args.segment)
         rms, rstats, _ = timed(pplan, make_step(pplan, "plain"), nst, all_kernels)
@@ -832,8 +832,8 @@ def main():
                      "kernel_ms_per_step": {k: rstats[k]["ms"] / nst for k in all_kernels},
                      "cg_iterations_applied": pplan.cg_applied()}
         pplan.close()
-        best = "recompute" if recompute["value"] > stored["value"] else "stored"
-        plain = dict((recompute if best == "recompute" else stored), variant=best, stored=stored,
+        best = "recompute" if recompute["value"] > default["value"] else "default"
+        plain = dict((recompute if best == "recompute" else default), variant=best, default=default,
                      recompute=recompute)
 
     # the precision form: the exact model with the readout DFTs as split-BF16 tcgen05
@@ -844,7 +844,7 @@ def main():
         xplan = mr.Plan(seq, form=mr.MRSTAT_FORM_SPLIT_BF16)
         nst = max(1, args.steps // 4)
         xms, xstats, _ = timed(xplan, make_step(xplan, "split"), nst, all_kernels)
-        # the encoding alone: forward (K1 + K2 + split x-DFT) and J^H w (split x-DFT^H + K4)
+        # forward and J^H w, whose readout DFTs are the split ones
         w_dev = torch.tensor(synth.random_kspace(seq.ntr, seq.nkx, 5), dtype=torch.complex64, device="cuda")
 
         def enc():
@@ -988,6 +988,8 @@ def main():
     per_launch = {k: stats[k]["ms"] / max(stats[k]["timed"], 1) for k in all_kernels}
     lowrank_like = args.form in ("lowrank", "surrogate")
     full_readout = nkx == nx
+    # the exact form's products re-run the recursion from states (hard pulses, no B1 map)
+    recomputed = args.form in ("plain", "split") and ny <= 256
     column_bytes = None
     max_trs_per_ky = int(np.bincount(np.mod(np.asarray(seq.ky), ny), minlength=ny).max())
     fft_y = full_readout and ny % 32 == 0 and ny // 32 <= 8
@@ -1025,10 +1027,18 @@ def main():
         # v and the phase 15, the adjoint phase and the four tangent products 17, the block
         # sums 2)
         work = {"jhw_dot": (86.0 * nv * ntr, "alu")}
-    elif full_readout and ny <= 256:
-        # one launch per product re-running the recursion: 41 multiply-adds (or half of one)
-        # per voxel-TR; the linearisation 21
+    elif args.form == "recompute":
+        # two launches per product: the rotation, the relaxations and the combination with the
+        # phase 67 flops per voxel-TR, and with the adjoint phase and tangent products 69
+        work = {"ycontract": (67.0 * nv * ntr, "alu"), "jhw_dot": (69.0 * nv * ntr, "alu")}
+    elif recomputed and full_readout:
+        # one launch per product re-running the recursion: 41 multiply-adds per voxel-TR; the
+        # linearisation 21
         work = {"jhw_dot": (2 * 41.0 * nv * ntr, "alu"), "bloch": (2 * 21.0 * nv * ntr, "alu")}
+    elif recomputed:
+        # J.v and Re(J^H w) apart, the readout DFT between them: 31 multiply-adds each
+        work = {"ycontract": (2 * 31.0 * nv * ntr, "alu"), "jhw_dot": (2 * 31.0 * nv * ntr, "alu"),
+                "bloch": (2 * 21.0 * nv * ntr, "alu")}
     else:
         work = {"jhw_dot": (d_bytes + ntr_pad * nx * 8 + nv * (8 + 4 + 16) + ntr_pad * 4, "hbm"),
                 "ycontract": (d_bytes + nv * 24 + ntr * nx * 8 + ntr_pad * 4, "hbm"),
@@ -1083,7 +1093,7 @@ def main():
            "xdft_adj": "tc_gemm.cu", "mlp_infer": "mlp.cu"}
     if lowrank_like:
         src.update({"jhw_dot": "lowrank.cu", "ycontract": "lowrank.cu"})
-    if args.form in ("plain", "split") and ny <= 256:
+    if recomputed:
         src.update({"jhw_dot": "recur.cu", "ycontract": "recur.cu", "bloch": "recur.cu"})
     if args.form == "recompute":
         src.update({"jhw_dot": "fused.cu"})
@@ -1204,10 +1214,16 @@ def main():
                      "recompute": f"plain FP32 form, recompute variant (Bloch recursion re-run in every product "
                                   f"from states every {args.segment} TRs, fused with the phase-encode sums)",
                      "split": "split-BF16 form (recursion re-run in every product, tcgen05 readout DFT)"}[args.form]
-        l2 = ("inputs larger than L2 (cached time courses %.0f MB)" % (d_bytes / 1e6) if not lowrank_like
-              else "L2 not flushed: the low-rank operands (~%.0f MB) are L2-resident by design; the "
-                   "linearisation streams the parameters and writes the coefficients each step"
-              % ((R * ny * 2 * nx * 2 * 2 + R * nkx * 2 * ny * 4 * 3) / 1e6))
+        if lowrank_like:
+            l2 = ("L2 not flushed: the low-rank operands (~%.0f MB) are L2-resident by design; the "
+                  "linearisation streams the parameters and writes the coefficients each step"
+                  % ((R * ny * 2 * nx * 2 * 2 + R * nkx * 2 * ny * 4 * 3) / 1e6))
+        elif recomputed or args.form == "recompute":
+            l2 = ("L2 not flushed: the products re-run the recursion from states and vectors of under "
+                  "%.0f MB, L2-resident by design; the linearisation rewrites them each step"
+                  % (nv * 4 * (6 + 6 * 8 + 4 * 4) / 1e6))
+        else:
+            l2 = "inputs larger than L2 (cached time courses %.0f MB)" % (d_bytes / 1e6)
         line = {"metric": METRIC, "value": value, "unit": "products/s", "n_gpus": world,
                 "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms,
                 "higher_is_better": True, "scaling": "weak", "vs_baseline": None,

@@ -111,10 +111,11 @@ typedef struct mrstat_plan_info_t {
  * Create a plan: validates the sequence, builds the per-TR rotation and phase
  * tables and allocates the small work buffers (x-DFT matrices, reduction scratch,
  * CG vectors).  The large buffers are allocated by the first call that needs them:
- * the time courses D (3 x ntr_padded x nv float32, 4 x with B1 estimated; filled by
- * mrstat_timecourses where the linearisation keeps states instead) by mrstat_linearize, the
- * m_y scratch (ntr_padded x nv float32) by mrstat_forward / mrstat_forward_ckpt.  Synchronises the current device once.  On failure *out is
- * set to NULL.  form: a mrstat_form, optionally | MRSTAT_ESTIMATE_B1.
+ * the time courses D (3 x ntr_padded x nv float32, 4 x with B1 estimated) and, where the
+ * linearisation keeps states instead, the states, by mrstat_linearize (which then goes without
+ * D where it does not fit: nothing of that form reads it), the m_y scratch (ntr_padded x nv
+ * float32) or states of m alone by mrstat_forward / mrstat_forward_ckpt.  Synchronises the
+ * current device once.  On failure *out is set to NULL.  form: a mrstat_form, optionally | MRSTAT_ESTIMATE_B1.
  * Errors: INVALID_ARG (null seq/out/arrays, bad form, non-finite or
  * negative flips, te/tr), SHAPE (sizes outside the ranges above, ky out of range),
  * OUT_OF_MEMORY, CUDA.
@@ -154,15 +155,17 @@ int mrstat_plan_inject_grid_stall(mrstat_plan* plan, int32_t block);
  * before up to eight segments of the train (the products re-run the recursion, as the
  * paper does inside every product: Algorithms 2 and 4), otherwise m_y and dm_y/dln T1,
  * dm_y/dln T2 at every echo; plus rho and the mask.  Both give the same products up to
- * float32 rounding.
+ * float32 rounding.  A stream-captured product replays the form of the linearisation it was
+ * captured with.
  *   alpha: device float [npar][nv] (see top; row 4 = B1 when B1 is estimated, and then
  *          a fourth channel dm_y/dB1 is cached).
  *   b1:    device float [nv] relative transmit field, or NULL for B1 = 1 (must be NULL
  *          when B1 is estimated).
  *   mask:  device uint8 [nv], nonzero = voxel takes part, or NULL for all voxels
  *          (Methods: voxels without significant proton density are excluded; a
- *          masked-out voxel contributes nothing to s and gets zero gradient).
- * Errors: INVALID_ARG (null plan/alpha, b1 given with B1 estimated), CUDA.
+ *          masked-out voxel contributes nothing to s and gets zero gradient, whatever
+ *          alpha and b1 hold there, NaN and infinities included).
+ * Errors: INVALID_ARG (null plan/alpha, b1 given with B1 estimated), OUT_OF_MEMORY, CUDA.
  */
 int mrstat_linearize(mrstat_plan* plan, const float* alpha, const float* b1,
                      const uint8_t* mask, void* stream);
@@ -192,8 +195,8 @@ int mrstat_jvp(mrstat_plan* plan, const float* v, float* jv, void* stream);
 int mrstat_jhw(mrstat_plan* plan, const float* w, float* g, void* stream);
 
 /*
- * Copy one time course channel of the linearisation out of the plan (a linearisation that
- * keeps states fills its time courses at the first such call): channel 0 = m_y, 1 =
+ * One time course channel of the linearisation (copied, or run again from the states of a
+ * linearisation that keeps those): channel 0 = m_y, 1 =
  * dm_y/dln T1, 2 = dm_y/dln T2 (3 = dm_y/dB1 when B1 is estimated) at every echo (the echo signal is i * m_y because
  * the RF phases 0/180 keep m_x = 0; Supporting Information S2).
  *   out: device float [ntr][nv].  Masked-out voxels read as 0.
@@ -229,8 +232,8 @@ int mrstat_set_recompute(mrstat_plan* plan, int32_t segment);
  * mrstat_jhw_ckpt then returns Re(J_s^H w) at that point by re-running each segment of
  * the recursion from its checkpoint (Supporting Information S2), all segments in
  * parallel, fused with the inner products of Algorithm 4; no time course is stored.
- * mrstat_jhw_ckpt reads alpha, b1 and mask from the caller's buffers given to the last
- * mrstat_forward_ckpt, which must still hold the same values.
+ * With a B1 map or ny > 256 mrstat_jhw_ckpt reads alpha, b1 and mask from the caller's buffers
+ * given to the last mrstat_forward_ckpt, which must still hold the same values.
  *   interval: positive multiple of 4 (64 is the usual choice).
  * Errors: INVALID_ARG, NOT_LINEARIZED (jhw_ckpt before forward_ckpt), OUT_OF_MEMORY, CUDA.
  */
@@ -266,7 +269,8 @@ int mrstat_jhjv(mrstat_plan* plan, const float* v, float* out, void* stream);
  *   NULL; U_out: device float [ntr][R]; sv_out: host double [R] singular values or NULL.
  *   1 <= R <= 32.  Allocates and frees its own work space; synchronises.
  * mrstat_lowrank_set_basis: adopts U (device float [ntr][R], R in {8, 16, 24, 32},
- *   orthonormal columns) and allocates the form's work space; synchronises.
+ *   orthonormal columns) and allocates the form's work space; synchronises.  A low-rank
+ *   linearisation with an earlier basis is dropped; an exact one stays.
  * mrstat_lowrank_linearize: makes the low-rank model at alpha the plan's linearisation
  *   for mrstat_jvp, mrstat_jhw, mrstat_jhjv and mrstat_cg_fixed.  coef = NULL projects
  *   the exact Bloch recursion onto U on the fly (no time course is stored); otherwise
@@ -487,8 +491,8 @@ int mrstat_cg_applied(mrstat_plan* plan, int32_t* applied);
  * ny = 32 N1 (N1 <= 8) and every image column's pair of blocks fits on the device at
  * once, each Steihaug solve is one persistent launch (the residual's product carries the
  * direction's by recurrence; the same decisions in exact arithmetic); if its grid waits
- * run out (2 s) the call returns TIMEOUT.  On return the plan holds the linearisation
- * at the returned alpha.
+ * run out (2 s) the call returns TIMEOUT.  On success the plan holds the linearisation
+ * at the returned alpha; a solve that fails once it has begun leaves none.
  *   d:      device float [ntr][nkx][2] measured k-space data.
  *   alpha:  device float [npar][nv], initial guess in, estimate out (B1 in row 4 when
  *           estimated; reflected into [b1_min, b1_max] like T1 and T2).

@@ -8,8 +8,9 @@ because alpha is real.
 With ``checkpoint=k`` (a multiple of 4, default 64) the forward keeps only the
 Bloch state of every voxel at every k-th TR and the backward re-runs the segments of
 the recursion from those states (mrstat_forward_ckpt / mrstat_jhw_ckpt); with
-``checkpoint=0`` the forward caches the full time courses and the backward streams
-them (mrstat_linearize / mrstat_jhw).  Both run entirely in libmrstat.
+``checkpoint=0`` the forward linearises and the backward takes the plan's own adjoint
+(mrstat_linearize / mrstat_jhw: states of up to eight segments, or the stored time
+courses with a B1 map or more than 256 rows).  Both run entirely in libmrstat.
 
 A plan holds the state of one forward at a time: call backward before the next
 forward on the same plan.

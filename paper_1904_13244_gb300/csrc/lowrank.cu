@@ -56,8 +56,10 @@ __device__ __forceinline__ void put_split_pair(__nv_bfloat16* hi, __nv_bfloat16*
 // E a and E b + D y with E = E2(TE), D = dE/dln T2, constants of the voxel that the finished
 // sums take; the relaxations over TE and TR - TE act as one step over TR.
 //
-// Bound by the FP32 pipe: 3 R multiply-adds of the projection (in packed pairs of basis
-// functions) and 21 of the recursion per voxel and TR, one voxel per thread.  The rows of U
+// Work: 3 R multiply-adds of the projection (in packed pairs of basis functions) and 21 of the
+// recursion per voxel and TR, one voxel per thread.  Bound by the few warps (6 per SM on
+// average): they issue on 59 % of the cycles and keep the FP32 pipe busy on 65 % while they
+// run, and the SMs idle for a quarter of the launch once their voxels are done.  The rows of U
 // and the pulse table come through shared memory two chunks deep (read from global memory
 // per TR, the pulse table alone cost an L2 latency every few TRs).  Blocks of two warps: a
 // block outside the mask ends at once, so the warps that count spread over the SMs.  At 224 x

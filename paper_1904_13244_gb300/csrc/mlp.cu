@@ -8,8 +8,8 @@
 // A tanh layer maps a tangent t to (1 - a^2) (W t); the tangents of u along ln T1 and
 // ln T2 are (1/s1, 0, 0) and (0, 1/s2, 0).  So a batch of B samples runs as M = 3B rows
 // (values, ln T1 tangents, ln T2 tangents) through every layer: one BF16 tcgen05 GEMM
-// per layer shared by the value and both tangent streams, float32 accumulation,
-// then one element-wise kernel for the activation and the tangent scaling.
+// per layer shared by the value and both tangent streams, float32 accumulation, the
+// activation and the tangent scaling in its epilogue.
 //
 // Training minimises the Sobolev loss
 //     L = 1/B sum_b sum_r [(c - c*)^2 + lam ((dc1 - dc1*)^2 + (dc2 - dc2*)^2)] / scale_r^2
@@ -99,15 +99,17 @@ __global__ void mlp_cast_kernel(const float* __restrict__ theta, int out, int in
 }
 
 // ---------------------------------------------------------------------------
-// Fused inference layer.  Per K chunk TMA brings the three 128-row tiles of the layer
-// input (value rows b, ln T1 tangent rows B + b, ln T2 tangent rows 2B + b) and one weight
-// tile; one thread issues three tcgen05.mma per K step into three TMEM accumulators, so
-// the epilogue sees z, z1, z2 of the same (sample, feature) and applies the layer there:
+// The layer kernel of inference and training (LayerMode).  Per K chunk TMA brings the three
+// 128-row tiles of the layer input (value rows b, ln T1 tangent rows B + b, ln T2 tangent rows
+// 2B + b) and one weight tile; one thread issues three tcgen05.mma per K step into three TMEM
+// accumulators, so the epilogue sees z, z1, z2 of the same (sample, feature) and applies the
+// layer there.  Inference:
 //   hidden: a = tanh(z + bias), s_k = (1 - a^2) z_k, written as the next layer's BF16 input;
 //   output: pred[k][r][b] = scale_r (z_k + [k = 0] bias_r), coalesced along the samples.
-// The pre-activations never reach global memory.  The hidden-layer tanh is the hardware
+// Its pre-activations never reach global memory, and its hidden-layer tanh is the hardware
 // tanh.approx.f32 (relative error about 2^-11, below the BF16 rounding of the values it
-// produces).
+// produces).  Training takes tanhf and keeps a, z1, z2 in float32 for the way back, which the
+// same kernel goes with the transposed weights.
 //
 __device__ __forceinline__ float tanh_fast(float x) {
   float y;
@@ -549,10 +551,12 @@ mlp_layer_persistent_kernel(const __grid_constant__ CUtensorMap tx, const __grid
 // rows: one CTA per 128 x 64 tile.  Both operands are read as they were written (rows = the
 // GEMM's K): MN-major tiles of 64 rows, so no transposed copies exist.  Bound by the chain
 // of dependent MMAs over the rows, about 75 ns per 16 rows at any tile size: 57 us at 4096
-// samples (108 us from transposed K-major copies, 64-row chunks of 32 KB).  The rows are not
-// split over CTAs: the tensor core's float32 accumulation rounds towards zero, so a split
-// changes a gradient by 3e-5 relative.  The launch uses few SMs (8 at H = 256), so the three
-// layers' gradients run on streams of their own beside the backward layers.
+// samples (108 us from transposed K-major copies, 64-row chunks of 32 KB); the tensor pipe is
+// active on 23 % of its SMs' cycles.  The rows are not split over CTAs by choice, not by need:
+// a trial with sixteen parts took 13 us, but the tensor core's float32 accumulation rounds
+// towards zero, so shorter chains change a gradient by 3e-5 relative (its error against
+// float64 is 1e-3, from the BF16 operands).  The launch uses few SMs (8 at H = 256), so the
+// three layers' gradients run on streams of their own beside the backward layers.
 // ---------------------------------------------------------------------------
 constexpr int kDwN = 64;                             // columns of a tile
 constexpr int kDwStages = 8;

@@ -29,12 +29,15 @@
 // adjoint, which needs no barrier): one barrier per chunk, the sums over the warps formed by every warp for itself.  The segments of a tile are
 // the blocks of a cluster and add their gradients through distributed shared memory.
 //
-// Bound by the FP32 pipe: 41 packed multiply-adds per row pair and TR for Re(J^H J) v (68 us
-// at 224 x 224, 1120 TRs), 31 for the half products; about 45 % of that pipe is reached with 14
-// warps per SM (128 registers each: the state, factors, coefficients and sums of four rows).
-// Measured at that size, against the stored time courses: linearisation 50 us (120-180),
-// J.v 92 (111 + 3), Re(J^H w) 92 (126), Re(J^H J) v 143 (241 in three launches), signal
-// 29 + 49 (73 + 3 + 68).  Tried: two columns per block (129 / 131 / 177 us: the phases serve
+// Work: 41 packed multiply-adds per row pair and TR for Re(J^H J) v (68 us of the FP32 pipe at
+// 224 x 224, 1120 TRs), 31 for the half products.  No single limit binds: counters show the
+// pipe busy on 52 % (Re(J^H J) v) to 59 % (J.v) of the cycles (a packed instruction holds it for
+// two) with 11-12 warps per SM, and the warps' stalls spread over the pipe (1.1-1.6 per
+// instruction issued), fixed latencies (1.3-1.4), the chunks' barriers (0.8-1.0) and shared
+// memory (0.3-0.9).  128 registers a thread (the state, factors, coefficients and sums of four
+// rows) allow two blocks per SM.  Measured at that size, against the stored time courses:
+// linearisation 50 us (120-180), J.v 92 (111 + 3), Re(J^H w) 92 (126), Re(J^H J) v 143 (241 in
+// three launches), signal 29 + 49 (73 + 3 + 68).  Tried: two columns per block (129 / 131 / 177 us: the phases serve
 // fewer threads), phases computed in the kernel instead of copied (106 / 103 / 158).
 #include <algorithm>
 

@@ -99,27 +99,28 @@ def test_lowrank_projection(with_b1, nx, ny, rank, value):
 
 
 @pytest.mark.parametrize("value", BAD)
+@pytest.mark.parametrize("rows", [slice(2, 4), slice(None)], ids=["rho", "every row"])
 @pytest.mark.parametrize("model", ["slice", "b1", "estimated b1", "checkpointed b1", "recompute"])
-def test_proton_density(model, value):
+def test_proton_density(model, rows, value):
     import paper_1904_13244_gb300 as mr
     seq, a, mask, v, w = make(29, 21, 4, extra=3, npar=5 if model == "estimated b1" else 4)
-    rows = slice(2, 4)
     b1 = 0.9 + 0.2 * torch.rand(seq.nv, device="cuda") if model in ("b1", "checkpointed b1") else None
     bad = spoil(a, mask, value, rows)
+    bad_b1 = spoil(b1[None], mask, value)[0] if b1 is not None and rows == slice(None) else b1
     with mr.Plan(seq, estimate_b1=model == "estimated b1") as plan:
         if model == "slice":
             plan.set_slice_profile(16, 6, 0.2, 4.0, 2.0)
         if model == "recompute":
             plan.set_recompute(32)
         outs = []
-        for x in (a, bad):
+        for x, b in ((a, b1), (bad, bad_b1)):
             if model == "checkpointed b1":
-                outs.append([plan.forward_ckpt(x, b1=b1, mask=mask, interval=16), plan.jhw_ckpt(w)])
+                outs.append([plan.forward_ckpt(x, b1=b, mask=mask, interval=16), plan.jhw_ckpt(w)])
             elif model == "recompute":
                 plan.linearize(x, mask=mask)
                 outs.append([plan.jvp(v), plan.jhw(w), plan.jhjv(v)])
             else:
-                outs.append(exact_calls(plan, x, mask, v, w, b1=b1))
+                outs.append(exact_calls(plan, x, mask, v, w, b1=b))
     assert all_equal(outs[1], outs[0])
 
 
