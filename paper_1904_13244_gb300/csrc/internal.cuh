@@ -249,6 +249,8 @@ int lowrank_setup(Plan* p, const float* U_dev, int R, cudaStream_t st);
 void lowrank_free(LowRank* L);
 cudaError_t lowrank_project(const Plan& p, const LowRank& L, const float* alpha, const float* b1,
                             const uint8_t* mask, float* coef, cudaStream_t st);
+// notes that a projection wrote L's coefficients on st
+void lowrank_projected(LowRank& L, cudaStream_t st);
 cudaError_t lowrank_adopt(Plan* p, const float* coef, cudaStream_t st);
 int lowrank_jvp(Plan* p, const float* v, float2* jv, cudaStream_t st);
 int lowrank_jhw(Plan* p, const float2* w, float* g, cudaStream_t st);

@@ -2535,14 +2535,35 @@ static int lowrank_jhjv_full_readout(Plan* p, const float* v, float* out, double
   return e == cudaSuccess ? MRSTAT_OK : cuda_fail(e, "low-rank J^H J v");
 }
 
-// The image-column copy of the coefficients, refreshed when they changed.
+// The stream capture st is recording into, 0 if none.
+static unsigned long long capture_id(cudaStream_t st) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if (cudaStreamGetCaptureInfo(st, &s, &id) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return s == cudaStreamCaptureStatusActive ? id : 0;
+}
+
+void lowrank_projected(LowRank& L, cudaStream_t st) {
+  L.coefT_dirty = true;
+  if (capture_id(st) != 0) L.coef_replayed = true;
+}
+
+// The image-column copy of the coefficients, refreshed when they changed.  What the host knows
+// holds only within one capture, or outside of any: a recorded product is replayed after other
+// linearisations, and a recorded projection changes the coefficients when it is replayed.
 static cudaError_t ensure_coef_columns(Plan* p, cudaStream_t st) {
   LowRank& L = *p->lr;
-  if (!L.coefT_dirty && L.coefT_src == L.coef) return cudaSuccess;
+  const unsigned long long id = capture_id(st);
+  if (!L.coefT_dirty && L.coefT_src == L.coef && L.coefT_capture == id && (id != 0 || !L.coef_replayed))
+    return cudaSuccess;
   const dim3 grid((p->nx + 31) / 32, (p->ny + 31) / 32, 3 * L.R);
   lr_coef_transpose_kernel<<<grid, dim3(32, 8), 0, st>>>(L.coef, p->nx, p->ny, L.coefT, nullptr);
   L.coefT_src = L.coef;
   L.coefT_dirty = false;
+  L.coefT_capture = id;
   return cudaGetLastError();
 }
 
@@ -2558,6 +2579,7 @@ cudaError_t lowrank_adopt(Plan* p, const float* coef, cudaStream_t st) {
   lr_coef_transpose_kernel<<<grid, dim3(32, 8), 0, st>>>(coef, p->nx, p->ny, L.coefT, L.coef);
   L.coefT_src = L.coef;
   L.coefT_dirty = false;
+  L.coefT_capture = capture_id(st);
   return cudaGetLastError();
 }
 

@@ -41,6 +41,8 @@ struct LowRank {
   float* coefT = nullptr;          // [3 R][nx][ny]: coef in image-column order (column kernel)
   const float* coefT_src = nullptr;  // the coef buffer coefT was made from
   bool coefT_dirty = true;         // coef changed in place since
+  unsigned long long coefT_capture = 0;  // the stream capture coefT was made in (0: none)
+  bool coef_replayed = false;      // a captured projection may change coef whenever it is replayed
   void *a1_hi = nullptr, *a1_lo = nullptr;    // [R ny][k1]   readout-DFT input rows
   void *a23_hi = nullptr, *a23_lo = nullptr;  // [R nkx][k23] phase-encode DFT input rows
   void *a4_hi = nullptr, *a4_lo = nullptr;    // [R ny][k4]   readout adjoint input rows

@@ -104,7 +104,7 @@ int mrstat_lowrank_linearize(mrstat_plan* plan_, const float* alpha, const float
   if (coef == nullptr) {
     Span sp(p, MRSTAT_K_BLOCH, st);
     e = lowrank_project(*p, L, alpha, b1, mask, L.coef, st);
-    L.coefT_dirty = true;
+    lowrank_projected(L, st);
   } else {
     e = lowrank_adopt(p, coef, st);
   }

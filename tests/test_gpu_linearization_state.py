@@ -83,3 +83,58 @@ def test_captured_calls_follow_the_linearisation():
         x.copy_(b)
         lin.replay()
         assert all(torch.equal(p, q) for p, q in zip(calls(), ref))
+
+
+def test_captured_lowrank_calls_follow_the_coefficients():
+    """The same for the low-rank form, whose column kernels read a reordered copy of the
+    coefficients: whatever was captured, a product sees those of the last linearisation."""
+    import paper_1904_13244_gb300 as mr
+    seq = synth.make_sequence(20, 64, 3, 7.6, 3.8, seed=1)
+    rng = np.random.default_rng(1)
+    a, b = (torch.tensor(np.stack([rng.uniform(np.log(300), np.log(3000), seq.nv),
+                                   rng.uniform(np.log(30), np.log(300), seq.nv), rng.uniform(0.5, 1, seq.nv),
+                                   rng.uniform(-1, 1, seq.nv)]), dtype=torch.float32, device="cuda") for _ in range(2))
+    U = torch.linalg.qr(torch.randn((seq.ntr, 16), generator=torch.Generator().manual_seed(3)))[0].contiguous().cuda()
+    v = torch.tensor(synth.random_params(seq.nv, 1), dtype=torch.float32, device="cuda")
+    with mr.Plan(seq) as plan:
+        plan.lowrank_set_basis(U)
+
+        def calls():
+            return [plan.jhjv(v), plan.jvp(v)]
+
+        ref, coef = [], []
+        for x in (a, b):
+            plan.lowrank_linearize(x)
+            coef.append(plan.lowrank_coefficients())
+            ref.append(calls())
+        assert not torch.equal(ref[0][0], ref[1][0])
+        x = a.clone()
+        torch.cuda.synchronize()
+        reads, proj, both = (torch.cuda.CUDAGraph() for _ in range(3))
+        with torch.cuda.graph(reads):
+            out = calls()
+        with torch.cuda.graph(proj):
+            plan.lowrank_linearize(x)
+        with torch.cuda.graph(both):
+            plan.lowrank_linearize(x, coef=coef[0])
+            out_both = calls()
+
+        def same(got, k):
+            return all(torch.equal(p, q) for p, q in zip(got, ref[k]))
+
+        plan.lowrank_linearize(a)
+        reads.replay()
+        assert same(out, 0)
+        plan.lowrank_linearize(b, coef=coef[1])
+        reads.replay()
+        assert same(out, 1)
+        proj.replay()  # an adopted linearisation, then a replayed projection (rho stays b's or x's)
+        assert same(calls(), 0)
+        x.copy_(b)
+        proj.replay()
+        assert same(calls(), 1)
+        reads.replay()
+        assert same(out, 1)
+        x.copy_(a)
+        both.replay()
+        assert same(out_both, 0) and same(calls(), 0)
